@@ -276,6 +276,15 @@ lbm_status lbm_set_graphs(lbm_ctx *ctx, int32_t enabled);
  * again when tuning is automatic.  Measured on one GB300: the 256-lattice
  * 256^2 CIL batch in FP32 at 85.9 GLUPS persistent (16-row strips) against
  * 81.3 per step; in FP16 storage the per-step launch stays faster (83.5).
+ * Mode 2 also considers, for a group whose lattices each fit the shared memory
+ * of a cluster of up to 16 blocks (both buffers with their halo rows; about 45
+ * thousand D2Q9 sites in FP32, twice that in 16-bit storage), the resident
+ * launch: one cluster per lattice keeps it on chip for a whole stretch of
+ * steps, reading and writing device memory once per stretch.  It is kept where
+ * it is faster than the forms above (measured: the paper's 90 x 30 MIPS box at
+ * 1.2 us per step against 12.4, 32 boxes of 180 x 60 at 6 us against 12);
+ * lbm_get_persistent reports 0 for such a group, and its sample steps and
+ * single steps launch once per step.  Modes 0 and 1 and fixed shapes never use it.
  * The waits are bounded (about 1 s, then the error flag is raised and the call
  * that reads it returns LBM_ERR_TIMEOUT).  Each launch first clears its
  * counters in the context's scratch (a memset on the bound stream; a graph

@@ -73,6 +73,11 @@ struct GroupHost {
     size_t persist_off = 0, persist_bytes = 0, pg_off = 0;
     int npg = 0;
     bool persist = false;  // mode 2: the tuner chose persistent launches for this group
+    // mode 2: the tuner chose the resident launch (whole lattices in the shared
+    // memory of clusters) for stretches of plain steps; its plan
+    bool resident = false;
+    int res_cluster = 0, res_threads = 0;
+    size_t res_smem = 0;
 };
 
 struct GraphKey {
@@ -507,11 +512,37 @@ cudaError_t launch_group_persistent(const lbm_ctx *c, const GroupHost &g, int sr
     return launch_persistent_bf16(g.model, g.vec, noise, a, p, g.blocks, g.warps, stream);
 }
 
+cudaError_t launch_resident(const GroupHost &g, const StepArgs &a, const ResidentArgs &p, int *clusters,
+                            cudaStream_t stream)
+{
+    if (g.storage == LBM_F32) return launch_resident_f32(g.q, g.model, a, p, clusters, stream);
+    if (g.storage == LBM_F16_SHIFTED) return launch_resident_f16(g.q, g.model, a, p, clusters, stream);
+    return launch_resident_bf16(g.q, g.model, a, p, clusters, stream);
+}
+
+// Whether a group runs stretches of plain steps as resident launches: where
+// the tuner chose them (mode 2).
+bool resident_ok(const lbm_ctx *c, const GroupHost &g) { return c->persist_mode == 2 && g.resident; }
+
+// m steps k .. k+m-1 of group g in one resident launch.
+cudaError_t launch_group_resident(const lbm_ctx *c, const GroupHost &g, int src, uint32_t k, int64_t m,
+                                  cudaStream_t stream, bool retime = false)
+{
+    ResidentArgs p;
+    p.dst = retime ? src ^ 1 : src ^ (int)(m & 1);
+    p.nsteps = (int)m;
+    p.cluster = g.res_cluster;
+    p.threads = g.res_threads;
+    p.smem = g.res_smem;
+    return launch_resident(g, step_args(c, g, src, k), p, nullptr, stream);
+}
+
 // The tuner's measure of a group: `steps` recomputations of the current step
 // into the spare buffer (the state is left as it was), as one persistent launch
 // in its timing form or as that many per-step launches.
 cudaError_t launch_group_timed(const lbm_ctx *c, const GroupHost &g, int steps, cudaStream_t stream)
 {
+    if (resident_ok(c, g)) return launch_group_resident(c, g, c->parity, 0, steps, stream, true);
     if (persistent_ok(c, g)) return launch_group_persistent(c, g, c->parity, 0, steps, stream, true);
     for (int q = 0; q < steps; ++q) {
         const cudaError_t e = launch_group_step(c, g, c->parity, 0, false, stream);
@@ -612,8 +643,8 @@ cudaError_t join_groups(lbm_ctx *c)
 // Enqueue n steps starting at host time t0 from buffer parity p0.  The steps
 // fall into runs without a sample step, each followed by its sample step (if
 // it lies within the n).  Per run, every group steps on its own stream (see
-// fork_groups): a group the persistent launch takes runs as few launches as its
-// step limit allows, any other launches once per step.  Then the sample step
+// fork_groups): a group the resident or the persistent launch takes runs as few
+// launches as the step limit allows, any other launches once per step.  Then the sample step
 // of every group, the join, and the finaliser.
 lbm_status enqueue_steps(lbm_ctx *c, int64_t n, int64_t t0, int p0, int64_t *launches)
 {
@@ -640,11 +671,15 @@ lbm_status enqueue_steps(lbm_ctx *c, int64_t n, int64_t t0, int p0, int64_t *lau
         if (par && !forked) CK(fork(), "fork launch groups");
         for (size_t gi = 0; gi < c->groups.size(); ++gi) {
             const GroupHost &g = c->groups[gi];
-            const int64_t mmax = persistent_ok(c, g) ? persist_steps_max(g) : 1;
+            const bool res = resident_ok(c, g);
+            const int64_t mmax = res ? PERSIST_STEPS_MAX : (persistent_ok(c, g) ? persist_steps_max(g) : 1);
             for (int64_t kk = k; kk < e;) {
                 const int64_t m = std::min(e - kk, mmax);
                 CK(prof_begin(c, true, m), "record event");
-                if (m >= 2)
+                if (m >= 2 && res)
+                    CK(launch_group_resident(c, g, (int)((p0 + kk) & 1), (uint32_t)kk, m, stream_of(gi)),
+                       "launch resident step kernel");
+                else if (m >= 2)
                     CK(launch_group_persistent(c, g, (int)((p0 + kk) & 1), (uint32_t)kk, m, stream_of(gi)),
                        "launch persistent step kernel");
                 else
@@ -738,8 +773,61 @@ struct EventPair {
 // the shape.
 struct Alt {
     Shape shape;
-    bool persist;
+    bool persist, resident;
 };
+
+// The resident launch's plan for a group: the cluster size (blocks per
+// lattice) with the least estimated time per step, if any fits.  A step takes
+// a latency (barrier, one pass of dependent arithmetic) plus the sites an SM
+// has to update, in waves of the clusters that fit the GPU at once.  In SM
+// cycles, RES_STEP_CYCLES and RES_SITE_CYCLES are the measured latency of a
+// step of a nearly empty band and the time per site of a full one.
+constexpr double RES_STEP_CYCLES = 1000.0, RES_SITE_CYCLES = 4.0;
+
+bool plan_resident(const lbm_ctx *c, GroupHost &g)
+{
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return false;
+    int min_ny = 1 << 30;
+    for (int m : g.members) min_ny = std::min(min_ny, c->lats[m].lat.ny);
+    const int nl = (int)g.members.size();
+    double best = 1e30;
+    long long prev_sites = -1;
+    for (int C = 1; C <= 16; ++C) {
+        if (min_ny / C < resident_halo(g.model)) break;
+        size_t smem = 0;
+        long long sites = 0;
+        for (int m : g.members) {
+            const lbm_lattice &l = c->lats[m].lat;
+            smem = std::max(smem, resident_smem_bytes(g.q, (int)elem_bytes(g.storage), g.model, l.nx, l.ny, C));
+            sites = std::max(sites, (long long)ceil_div(l.ny, C) * l.nx);
+        }
+        if (smem > STAGED_SMEM_MAX || sites == prev_sites) continue;  // too large, or no less work per block
+        prev_sites = sites;
+        const int passes = ceil_div(sites, RESIDENT_THREADS);
+        ResidentArgs p;
+        p.dst = 0;
+        p.nsteps = 1;
+        p.cluster = C;
+        p.threads = ceil_div(ceil_div(sites, passes), 32) * 32;
+        p.smem = smem;
+        int active = 0;
+        if (launch_resident(g, step_args(c, g, 0, 0), p, &active, c->stream) != cudaSuccess || active < 1) {
+            cudaGetLastError();  // this device cannot hold such a cluster
+            continue;
+        }
+        const int waves = ceil_div(nl, active), per_sm = ceil_div((long long)std::min(nl, active) * C, sms);
+        const double t = waves * (RES_STEP_CYCLES + per_sm * RES_SITE_CYCLES * (double)sites);
+        if (t < best) {
+            best = t;
+            g.res_cluster = C;
+            g.res_threads = p.threads;
+            g.res_smem = smem;
+        }
+    }
+    return best < 1e29;
+}
 
 lbm_status tune_group(lbm_ctx *c, GroupHost &g, std::vector<Alt> *alts)
 {
@@ -783,6 +871,23 @@ lbm_status tune_group(lbm_ctx *c, GroupHost &g, std::vector<Alt> *alts)
     float best = 1e30f, best_kind[2] = {1e30f, 1e30f}, best_step = 1e30f;
     Shape bs{g.vec, g.rows, g.warps, g.stages}, bk[2] = {bs, bs}, bstep = bs;
     bool bp = g.persist, bkp[2] = {bp, bp};
+    // The time of `steps` steps in the group's current shape and form, scaled
+    // to TUNE_STEPS (steps grow until the timing is long enough).
+    auto time_form = [&](int steps, float *out) -> lbm_status {
+        float ms = 0.f;
+        while (true) {
+            CK(cudaEventRecord(e0, c->stream), "record event");
+            CK(launch_group_timed(c, g, steps, c->stream), "tuning launch");
+            CK(cudaEventRecord(e1, c->stream), "record event");
+            CK(cudaEventSynchronize(e1), "synchronise event");
+            CK(cudaEventElapsedTime(&ms, e0, e1), "event time");
+            if (ms >= TUNE_MIN_MS || steps >= TUNE_STEPS_MAX) break;
+            steps = std::min(TUNE_STEPS_MAX, (int)std::ceil(steps * TUNE_MIN_MS / std::max(ms, 1e-3f)) + 1);
+        }
+        *out = ms * (float)TUNE_STEPS / (float)steps;
+        return LBM_OK;
+    };
+    g.resident = false;
     for (const Shape &sh : cands) {
         g.vec = sh.vec;
         g.rows = sh.rows;
@@ -801,18 +906,9 @@ lbm_status tune_group(lbm_ctx *c, GroupHost &g, std::vector<Alt> *alts)
                 cudaGetLastError();
                 continue;
             }
-            int steps = persistent_ok(c, g) ? TUNE_STEPS_PERSIST : TUNE_STEPS;
             float ms = 0.f;
-            while (true) {
-                CK(cudaEventRecord(e0, c->stream), "record event");
-                CK(launch_group_timed(c, g, steps, c->stream), "tuning launch");
-                CK(cudaEventRecord(e1, c->stream), "record event");
-                CK(cudaEventSynchronize(e1), "synchronise event");
-                CK(cudaEventElapsedTime(&ms, e0, e1), "event time");
-                if (ms >= TUNE_MIN_MS || steps >= TUNE_STEPS_MAX) break;
-                steps = std::min(TUNE_STEPS_MAX, (int)std::ceil(steps * TUNE_MIN_MS / std::max(ms, 1e-3f)) + 1);
-            }
-            ms *= (float)TUNE_STEPS / (float)steps;  // per TUNE_STEPS steps
+            st = time_form(persistent_ok(c, g) ? TUNE_STEPS_PERSIST : TUNE_STEPS, &ms);
+            if (st != LBM_OK) return st;
             if (ms < best) {
                 best = ms;
                 bs = sh;
@@ -832,11 +928,33 @@ lbm_status tune_group(lbm_ctx *c, GroupHost &g, std::vector<Alt> *alts)
     }
     const int other = bs.stages > 0 ? 0 : 1;
     alts->clear();
-    if (best_kind[other] < 1e29f) alts->push_back({bk[other], bkp[other]});
+    if (best_kind[other] < 1e29f) alts->push_back({bk[other], bkp[other], false});
     // mode 2, a persistent choice: its best per-step direct form too (beside
     // other groups, a persistent launch holds the SMs its grid fills; the best
     // staged form is the alternative above)
-    if (bp && best_step < 1e29f && bstep.stages == 0) alts->push_back({bstep, false});
+    if (bp && best_step < 1e29f && bstep.stages == 0) alts->push_back({bstep, false, false});
+    // mode 2: the resident launch where the lattices fit on chip and it is
+    // faster than the best of the others; single and sample steps then take the
+    // best per-step shape
+    bool res = false;
+    g.persist = false;
+    if (c->persist_mode == 2 && best_step < 1e29f && plan_resident(c, g)) {
+        g.resident = true;
+        float ms = 0.f;
+        lbm_status st = LBM_OK;
+        if (launch_group_timed(c, g, 1, c->stream) == cudaSuccess)
+            st = time_form(TUNE_STEPS_PERSIST, &ms);
+        else
+            cudaGetLastError(), ms = 1e30f;
+        if (st != LBM_OK) return st;
+        res = ms < best;
+    }
+    if (res) {
+        alts->push_back({bs, bp, false});
+        bs = bstep;
+        bp = false;
+    }
+    g.resident = res;
     g.vec = bs.vec;
     g.rows = bs.rows;
     g.warps = bs.warps;
@@ -913,9 +1031,10 @@ lbm_status do_tune(lbm_ctx *c)
             GroupHost &g = c->groups[gi];
             for (const Alt &al : alts[gi]) {
                 const Shape keep{g.vec, g.rows, g.warps, g.stages};
-                const bool keep_persist = g.persist;
+                const bool keep_persist = g.persist, keep_resident = g.resident;
                 set_shape(g, al.shape);
                 g.persist = al.persist;
+                g.resident = al.resident;
                 float ms = 0.f;
                 st = time_joint_step(c, &ms);
                 if (st != LBM_OK) return st;
@@ -924,6 +1043,7 @@ lbm_status do_tune(lbm_ctx *c)
                 } else {
                     set_shape(g, keep);
                     g.persist = keep_persist;
+                    g.resident = keep_resident;
                 }
             }
         }
@@ -1486,6 +1606,7 @@ lbm_status lbm_set_tuning(lbm_ctx *c, int32_t mode, int32_t vec, int32_t rows, i
         g.rows = rows;
         g.warps = warps;
         g.stages = stages;
+        g.resident = false;
     }
     c->tune_mode = 1;
     c->tuned = true;
@@ -1538,7 +1659,7 @@ lbm_status lbm_set_persistent(lbm_ctx *c, int32_t mode, int32_t l2_group_mib)
         return fail(c, LBM_ERR_INVALID_ARG, "l2_group_mib must be in [0, 2^20]");
     c->persist_mode = mode;
     c->persist_l2_mib = l2_group_mib;
-    for (auto &g : c->groups) g.persist = false;
+    for (auto &g : c->groups) g.persist = g.resident = false;
     if (mode == 2 && c->tune_mode == 0) c->tuned = false;  // the next lbm_step tunes, and chooses
     drop_graphs(c);
     if (c->bound) return upload_descs(c);

@@ -155,6 +155,33 @@ struct PersistArgs {
                      // current buffer into the spare one, so the state is left as it was
 };
 
+// The resident launch (lbm_step_resident.cuh): one cluster per lattice holds it in
+// shared memory for many steps.
+struct ResidentArgs {
+    int dst;      // buffer the last step writes (the first reads StepArgs::src; they may be the same)
+    int nsteps;
+    int cluster;  // blocks per cluster; every lattice has at least resident_halo rows per block
+    int threads;
+    size_t smem;  // dynamic shared memory per block (resident_smem_bytes of the largest lattice)
+};
+// Threads per block at most, and so the register cap (65536 / 768 = 85): one site
+// per thread needs 60 to 80 registers, and 24 warps per SM hide the latency of
+// the dependent arithmetic where a band gives each thread several sites.
+constexpr int RESIDENT_THREADS = 768;
+// Halo rows above and below a block's band: MIPS takes the density one row out.
+__host__ __device__ constexpr int resident_halo(int model) { return model == MODEL_MIPS ? 2 : 1; }
+// Where the MIPS densities start: after the two buffers of q planes.
+__host__ __device__ constexpr size_t resident_rho_offset(int q, int elem_bytes, size_t plane)
+{
+    return (2 * (size_t)q * plane * (size_t)elem_bytes + 15) / 16 * 16;
+}
+constexpr size_t resident_smem_bytes(int q, int elem_bytes, int model, int nx, int ny, int cluster)
+{
+    const size_t rows = ((size_t)ny + cluster - 1) / cluster, np = (size_t)nx + 2;
+    const size_t b = resident_rho_offset(q, elem_bytes, (rows + 2 * resident_halo(model)) * np);
+    return model == MODEL_MIPS ? b + (rows + 2) * np * 4 : b;
+}
+
 // ---------------------------------------------------------------------------
 // Philox4x32-10 (Salmon, Moraes, Dror, Shaw, SC'11): ten rounds of two 32x32
 // -> 64-bit products of counter words 0 and 2, whose high halves are XORed

@@ -29,6 +29,14 @@ cudaError_t launch_persistent_q7_f16(int model, int vec, int noise, const StepAr
                                      int step_blocks, int warps, cudaStream_t stream);
 cudaError_t launch_persistent_q7_bf16(int model, int vec, int noise, const StepArgs &a, const PersistArgs &p,
                                       int step_blocks, int warps, cudaStream_t stream);
+// the resident launch of small lattices (lbm_step_resident.cuh), q = 9 or 7;
+// with `clusters`, only reports how many clusters the GPU holds at once
+cudaError_t launch_resident_f32(int q, int model, const StepArgs &a, const ResidentArgs &p, int *clusters,
+                                cudaStream_t stream);
+cudaError_t launch_resident_f16(int q, int model, const StepArgs &a, const ResidentArgs &p, int *clusters,
+                                cudaStream_t stream);
+cudaError_t launch_resident_bf16(int q, int model, const StepArgs &a, const ResidentArgs &p, int *clusters,
+                                 cudaStream_t stream);
 cudaError_t launch_observe_f32(int vec, const StepArgs &a, int blocks, int warps, cudaStream_t stream);
 cudaError_t launch_observe_f16(int vec, const StepArgs &a, int blocks, int warps, cudaStream_t stream);
 cudaError_t launch_observe_bf16(int vec, const StepArgs &a, int blocks, int warps, cudaStream_t stream);
