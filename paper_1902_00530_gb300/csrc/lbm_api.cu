@@ -27,7 +27,8 @@ using namespace lbm;
 namespace {
 
 constexpr int ROWS_MIN = 8;        // smallest strip height; scratch is sized for it
-constexpr int CHUNK_COLS = 256;    // columns / rows / strips per finaliser block
+constexpr int CHUNK_LINES = 32;    // columns / rows per finaliser block ...
+constexpr int CHUNK_STRIPS = 256;  // ... and strips
 constexpr int NCHUNK_MAX = 1024;
 constexpr int GRAPH_CHUNK_MAX = 256;
 constexpr int PERSIST_STEPS_MAX = 4096;  // steps of one persistent launch
@@ -126,6 +127,7 @@ struct lbm_ctx {
     // joined back into the bound stream (parallel branches of the step graph)
     std::vector<cudaStream_t> aux;
     std::vector<cudaEvent_t> aux_ev;  // [0]: fork, [1 + i]: join of aux[i]
+    double *pinned = nullptr;         // see ensure_pinned
 };
 
 namespace {
@@ -233,6 +235,12 @@ int default_vec(const lbm_ctx *c, const GroupHost &g)
     return 1;
 }
 
+// Finaliser blocks of a lattice cut into nstrip strips.
+int chunks(const lbm_lattice &l, long long nstrip)
+{
+    return std::min(NCHUNK_MAX, std::max(ceil_div(std::max(l.nx, l.ny), CHUNK_LINES), ceil_div(nstrip, CHUNK_STRIPS)));
+}
+
 // Scratch / state layout; depends only on the lattices and sampling settings.
 void layout(lbm_ctx *c)
 {
@@ -246,7 +254,7 @@ void layout(lbm_ctx *c)
     }
     c->state_bytes = so;
     const int nl = (int)c->lats.size();
-    size_t o = 256;  // [0]: t (uint32), [4]: error flag (uint32)
+    size_t o = 256;  // [0]: t (uint32), [4]: error flag, [8]: the finaliser's count of lattices
     for (auto &L : c->lats) {
         L.ctr_off = o;
         o += 16;
@@ -278,8 +286,7 @@ void layout(lbm_ctx *c)
         const int nsx_max = ceil_div(L.lat.nx, 32);
         const int nsy_max = ceil_div(L.lat.ny, ROWS_MIN);
         const long long nstrip_max = (long long)nsx_max * nsy_max;
-        L.nchunk_max = std::min(NCHUNK_MAX,
-                                std::max(1, ceil_div(std::max<long long>({L.lat.nx, L.lat.ny, nstrip_max}), CHUNK_COLS)));
+        L.nchunk_max = chunks(L.lat, nstrip_max);
         L.scal_off = o;
         o = align256(o + nstrip_max * 5 * sizeof(double));
         L.colp_off = o;
@@ -334,7 +341,7 @@ LatDesc make_desc(const lbm_ctx *c, const LatHost &L, int block_begin, const Gro
     d.q = L.q;
     d.prog_off = L.prog_off;
     const long long nstrip = (long long)d.nsx * d.nsy;
-    d.nchunk = std::min(L.nchunk_max, std::max(1, ceil_div(std::max<long long>({L.lat.nx, L.lat.ny, nstrip}), CHUNK_COLS)));
+    d.nchunk = std::min(L.nchunk_max, chunks(L.lat, nstrip));
     // 1/tau in FP32 such that 1 - 1/tau is exact too (the noisy update weighs f*
     // by 1 - 1/tau and f^SS by 1/tau): automatic for 1/tau in [1/2, 2]
     // (Sterbenz); below 1/2 the value is rounded to a multiple of 2^-24.
@@ -701,7 +708,7 @@ lbm_status enqueue_steps(lbm_ctx *c, int64_t n, int64_t t0, int p0, int64_t *lau
             if (par) CK(join(), "join launch groups");
             CK(prof_begin(c, false), "record event");
             CK(launch_finalize(all_desc(c), (int)c->lats.size(), c->max_chunk, t_dev(c), (uint32_t)e, 1,
-                               err_dev(c), c->stream),
+                               err_dev(c), 0, nullptr, c->stream),
                "launch finaliser");
             CK(prof_end(c), "record event");
             ++*launches;
@@ -734,6 +741,14 @@ lbm_status read_error_flag(lbm_ctx *c)
         if (flag & DEVERR_TIMEOUT) return fail(c, LBM_ERR_TIMEOUT, "a device-side wait timed out");
         return fail(c, LBM_ERR_NUMERIC, "non-finite observable sums");
     }
+    return LBM_OK;
+}
+
+// The context's pinned host words (created once, freed by lbm_destroy), which
+// the finaliser writes: a record and the error word.
+lbm_status ensure_pinned(lbm_ctx *c)
+{
+    if (!c->pinned) CK(cudaMallocHost(reinterpret_cast<void **>(&c->pinned), 16 * sizeof(double)), "pinned host memory");
     return LBM_OK;
 }
 
@@ -1287,14 +1302,14 @@ lbm_status lbm_observables(lbm_ctx *c, int32_t lattice, lbm_obs *out)
     if (lattice < 0 || lattice >= (int32_t)c->lats.size() || !out)
         return fail(c, LBM_ERR_INVALID_ARG, "bad lattice index or null output");
     for (const GroupHost &g : c->groups) CK(launch_group_observe(c, g, c->parity), "launch observe kernel");
-    CK(launch_finalize(all_desc(c), (int)c->lats.size(), c->max_chunk, t_dev(c), 0, 0, err_dev(c), c->stream),
+    // the finaliser writes the record and the error word to the pinned words
+    st = ensure_pinned(c);
+    if (st != LBM_OK) return st;
+    CK(launch_finalize(all_desc(c), (int)c->lats.size(), c->max_chunk, t_dev(c), 0, 0, err_dev(c), lattice, c->pinned,
+                       c->stream),
        "launch finaliser");
-    double rec[8];
-    CK(cudaMemcpyAsync(rec, c->scratch + c->lats[lattice].now_off, sizeof(rec), cudaMemcpyDeviceToHost, c->stream),
-       "read observables");
     CK(cudaStreamSynchronize(c->stream), "synchronise");
-    long long tt;
-    std::memcpy(&tt, &rec[0], sizeof(tt));
+    const volatile double *rec = c->pinned;
     out->t = c->t;
     out->mass = rec[1];
     out->phi = rec[2];
@@ -1302,7 +1317,7 @@ lbm_status lbm_observables(lbm_ctx *c, int32_t lattice, lbm_obs *out)
     out->drho_x = rec[4];
     out->var_rho = rec[5];
     out->zeta = rec[6];
-    return read_error_flag(c);
+    return rec[8] != 0.0 ? read_error_flag(c) : LBM_OK;
 }
 
 lbm_status lbm_observable_series(lbm_ctx *c, int32_t lattice, lbm_obs *out, int32_t cap, int32_t *n_out)
@@ -1726,6 +1741,7 @@ void lbm_destroy(lbm_ctx *c)
     for (cudaEvent_t e : c->ev_pool) cudaEventDestroy(e);
     for (cudaEvent_t e : c->aux_ev) cudaEventDestroy(e);
     for (cudaStream_t s : c->aux) cudaStreamDestroy(s);
+    if (c->pinned) cudaFreeHost(c->pinned);
     delete c;
 }
 

@@ -336,6 +336,28 @@ __device__ __forceinline__ void load_vec(const typename Store<ST>::T *p, float s
     }
 }
 
+// The two halves of load_vec apart (at most 16 bytes): the raw word, which a
+// prefetch holds in the storage type's registers, and its expansion.
+template <int ST, int VEC> using RawVec = typename VecWord<(int)sizeof(typename Store<ST>::T) * VEC>::T;
+template <int ST, int VEC>
+__device__ __forceinline__ RawVec<ST, VEC> load_raw(const typename Store<ST>::T *p)
+{
+    return __ldg(reinterpret_cast<const RawVec<ST, VEC> *>(p));
+}
+template <int ST, int VEC>
+__device__ __forceinline__ void expand_raw(RawVec<ST, VEC> w, float shift, float out[VEC])
+{
+    using T = typename Store<ST>::T;
+    static_assert(sizeof(T) * VEC <= 16, "vector wider than 16 bytes");
+    if constexpr (sizeof(T) == 2 && VEC % 2 == 0) {
+        unpack_words<ST, VEC>(reinterpret_cast<const uint32_t *>(&w), shift, out);
+    } else {
+        const T *e = reinterpret_cast<const T *>(&w);
+#pragma unroll
+        for (int j = 0; j < VEC; ++j) out[j] = Store<ST>::get(e[j], shift);
+    }
+}
+
 // The same from any address space (shared memory): a plain vector load.
 template <int ST, int VEC>
 __device__ __forceinline__ void load_vec_plain(const typename Store<ST>::T *p, float shift, float out[VEC])

@@ -535,50 +535,113 @@ __device__ __forceinline__ void mips_gradients(const float rm[VEC + 2], const fl
     }
 }
 
-// Observable sums of one stored row (sites x0..x0+VEC-1) from its moments
-// rho and j = rho u: per-thread FP64 accumulators for the strip's column sums
-// and five scalar sums, and the row's density total reduced over the warp.
-// The sums that cancel (rho and rho^2 in the variance, j in the polar order of
-// a nearly disordered state) are formed in FP64 from the lane's first site on
-// (rho^2 exactly: a product of two FP32 values fits FP64), so they do not
-// depend on how the launch shape groups sites into lanes beyond FP64 rounding;
-// |j|, a sum of magnitudes, is summed in FP32 over the lane's sites.
-// Lattice-independent.
+// ---------------------------------------------------------------------------
+// Observable sums.  The sums that cancel (rho and rho^2 in the variance, j in
+// the polar order of a nearly disordered state) must not depend on how the
+// launch shape groups sites into lanes, so they are exact to FP64 rounding from
+// a lane's first site on.  FP64 itself is far too slow for that here: a GB300
+// SM issues about 2 FP64 lane operations per cycle, and five FP64 additions, four
+// conversions and the FP64 row reduction per site made a 4096^2 reduction 380 us
+// (0.14 sites per cycle and SM) where its bytes take 45 to 90 us.  A lane's
+// sums are therefore unevaluated FP32 pairs h + l (48 bits: 24 bits of a
+// value leave room for 2^24 values of one magnitude; a lane adds at most a
+// few thousand, so its sums are the exact ones), added with Knuth's TwoSum and
+// turned into FP64 once per strip; what joins strips is FP64 as before.
+// ---------------------------------------------------------------------------
+struct Pair {
+    float h, l;
+};
+// a = round(a + x); returns the rounding error, exactly
+__device__ __forceinline__ float two_sum(float &a, float x)
+{
+    const float s = __fadd_rn(a, x), b = __fsub_rn(s, a);
+    const float e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, b)), __fsub_rn(x, b));
+    a = s;
+    return e;
+}
+// a += x, exactly but for the rounding of the low word
+__device__ __forceinline__ void pair_add(Pair &a, float x)
+{
+    const float e = two_sum(a.h, x);
+    a.l = __fadd_rn(a.l, e);
+}
+__device__ __forceinline__ void pair_add(Pair &a, Pair x)
+{
+    const float l = __fadd_rn(a.l, x.l);
+    a.l = l;
+    pair_add(a, x.h);
+}
+__device__ __forceinline__ double pair_value(Pair a) { return (double)a.h + (double)a.l; }
+// The sum over the warp, in every lane.
+__device__ __forceinline__ Pair pair_warp_sum(Pair a)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) pair_add(a, Pair{__shfl_xor_sync(FULL, a.h, o), __shfl_xor_sync(FULL, a.l, o)});
+    return a;
+}
+
+// A lane's sums over its strip.  rho^2 = p + fma(r, r, -p) has 48 bits itself,
+// and the variance is the small difference of two such sums, so its sum is three
+// words (h + l + m).  That holds where p and its error stay in FP32's range
+// (2^-50 < rho < 2^60); rows with a density outside (an empty site, an absurd
+// scale) go to the FP64 sum r2d.
+template <int VEC> struct ObserveSums {
+    Pair col[VEC], jx, jy, r2, aj;
+    float r2m;
+    double r2d;
+    __device__ __forceinline__ void clear()
+    {
+#pragma unroll
+        for (int j = 0; j < VEC; ++j) col[j] = Pair{0.f, 0.f};
+        jx = jy = r2 = aj = Pair{0.f, 0.f};
+        r2m = 0.f;
+        r2d = 0.0;
+    }
+};
+
+// Add one stored row (sites x0..x0+VEC-1) from its moments rho and j = rho u,
+// and write the row's density total over the warp.  |j|, a sum of magnitudes,
+// is summed in FP32 over the lane's sites of the row.  Lattice-independent.
 template <int VEC>
 __device__ __forceinline__ void observe_moments(const float rv[VEC], const float jxv[VEC], const float jyv[VEC],
-                                                bool valid, double col[VEC], double acc[5], double *row_out,
-                                                int lane)
+                                                bool valid, ObserveSums<VEC> &o, double *row_out, int lane)
 {
-    double rs = 0.0, jxs = 0.0, jys = 0.0, r2s = 0.0;
-    float js = 0.f;
+    Pair rs{0.f, 0.f};
     if (valid) {
+        float js = 0.f;
+        bool in_range = true;
 #pragma unroll
         for (int j = 0; j < VEC; ++j) {
-            const float jx = jxv[j], jy = jyv[j];
-            const double r = (double)rv[j];
-            col[j] += r;
-            rs += r;
-            jxs += (double)jx;
-            jys += (double)jy;
-            r2s = __fma_rn(r, r, r2s);
+            const float r = rv[j], jx = jxv[j], jy = jyv[j];
+            pair_add(o.col[j], r);
+            pair_add(o.jx, jx);
+            pair_add(o.jy, jy);
+            in_range = in_range && r > 0x1p-50f && r < 0x1p60f;
             js += sqrtf(jx * jx + jy * jy);
+            if (j == 0) rs.h = r;
+            else pair_add(rs, r);
+        }
+        pair_add(o.aj, js);
+        if (in_range) {
+#pragma unroll
+            for (int j = 0; j < VEC; ++j) {
+                const float p = __fmul_rn(rv[j], rv[j]);
+                const float e = __fmaf_rn(rv[j], rv[j], -p), c = two_sum(o.r2.h, p);
+                o.r2m = __fadd_rn(o.r2m, __fadd_rn(two_sum(o.r2.l, c), two_sum(o.r2.l, e)));
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < VEC; ++j) o.r2d = __fma_rn((double)rv[j], (double)rv[j], o.r2d);
         }
     }
-    acc[0] += rs;
-    acc[1] += jxs;
-    acc[2] += jys;
-    acc[3] += r2s;
-    acc[4] += (double)js;
-    double t = rs;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(FULL, t, o);
-    if (lane == 0) *row_out = t;
+    rs = pair_warp_sum(rs);
+    if (lane == 0) *row_out = pair_value(rs);
 }
 
 // The same for a stored D2Q9 row.
 template <int VEC>
-__device__ __forceinline__ void observe_row(const float g[9][VEC], bool valid, double col[VEC],
-                                            double acc[5], double *row_out, int lane)
+__device__ __forceinline__ void observe_row(const float g[9][VEC], bool valid, ObserveSums<VEC> &o, double *row_out,
+                                            int lane)
 {
     float rv[VEC], jxv[VEC], jyv[VEC];
 #pragma unroll
@@ -587,26 +650,33 @@ __device__ __forceinline__ void observe_row(const float g[9][VEC], bool valid, d
         jxv[j] = (g[1][j] + g[5][j] + g[8][j]) - (g[3][j] + g[6][j] + g[7][j]);
         jyv[j] = (g[2][j] + g[5][j] + g[6][j]) - (g[4][j] + g[7][j] + g[8][j]);
     }
-    observe_moments<VEC>(rv, jxv, jyv, valid, col, acc, row_out, lane);
+    observe_moments<VEC>(rv, jxv, jyv, valid, o, row_out, lane);
 }
 
+// Write the strip's column sums and its five scalar sums (rho, j_x, j_y, rho^2,
+// |j|).
 template <int VEC>
 __device__ __forceinline__ void observe_flush(double *colp, double *scal, int nx, int s, int sy, int x0,
-                                              bool valid, const double col[VEC], double acc[5],
-                                              int lane)
+                                              bool valid, const ObserveSums<VEC> &o, int lane)
 {
+    Pair rho{0.f, 0.f};
+#pragma unroll
+    for (int j = 0; j < VEC; ++j) pair_add(rho, o.col[j]);
     if (valid) {
 #pragma unroll
-        for (int j = 0; j < VEC; ++j) colp[(size_t)sy * nx + x0 + j] = col[j];
+        for (int j = 0; j < VEC; ++j) colp[(size_t)sy * nx + x0 + j] = pair_value(o.col[j]);
     }
+    const Pair v[4] = {pair_warp_sum(rho), pair_warp_sum(o.jx), pair_warp_sum(o.jy), pair_warp_sum(o.aj)};
+    double r2 = (pair_value(o.r2) + (double)o.r2m) + o.r2d;
 #pragma unroll
-    for (int q = 0; q < 5; ++q) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc[q] += __shfl_xor_sync(FULL, acc[q], o);
-    }
+    for (int q = 16; q > 0; q >>= 1) r2 += __shfl_xor_sync(FULL, r2, q);
     if (lane == 0) {
-#pragma unroll
-        for (int q = 0; q < 5; ++q) scal[(size_t)s * 5 + q] = acc[q];
+        double *out = scal + (size_t)s * 5;
+        out[0] = pair_value(v[0]);
+        out[1] = pair_value(v[1]);
+        out[2] = pair_value(v[2]);
+        out[3] = r2;
+        out[4] = pair_value(v[3]);
     }
 }
 
@@ -662,13 +732,8 @@ __device__ __forceinline__ void direct_strip(const StepArgs &a, const LatDesc *d
     const uint32_t id = (uint32_t)dp->id;
     const bool noise = NOISE == 2 ? d.sigma_q > 0.f : NOISE == 1;
 
-    double col[VEC], acc[5];
-    if constexpr (SAMPLE) {
-#pragma unroll
-        for (int j = 0; j < VEC; ++j) col[j] = 0.0;
-#pragma unroll
-        for (int q = 0; q < 5; ++q) acc[q] = 0.0;
-    }
+    ObserveSums<VEC> obs;
+    if constexpr (SAMPLE) obs.clear();
 
     // MIPS: the densities of rows y-1 and y slide along in registers; the
     // populations of row y are pulled again when row y is updated (they were
@@ -740,7 +805,7 @@ __device__ __forceinline__ void direct_strip(const StepArgs &a, const LatDesc *d
 #pragma unroll
                 for (int j = 0; j < VEC; ++j)
                     g[i][j] = Store<ST>::get(Store<ST>::put(out[i][j], sh.q9(i)), sh.q9(i));
-            observe_row<VEC>(g, valid, col, acc, dp->rowp + (size_t)sx * ny + y, lane);
+            observe_row<VEC>(g, valid, obs, dp->rowp + (size_t)sx * ny + y, lane);
         }
         if constexpr (MODEL == MODEL_MIPS) {
 #pragma unroll
@@ -750,7 +815,7 @@ __device__ __forceinline__ void direct_strip(const StepArgs &a, const LatDesc *d
             }
         }
     }
-    if constexpr (SAMPLE) observe_flush<VEC>(dp->colp, dp->scal, nx, s, sy, x0, valid, col, acc, lane);
+    if constexpr (SAMPLE) observe_flush<VEC>(dp->colp, dp->scal, nx, s, sy, x0, valid, obs, lane);
 }
 
 template <int MODEL, int ST, int VEC, bool SAMPLE, int NOISE>
@@ -792,25 +857,31 @@ __global__ void __launch_bounds__(256) observe_kernel(const StepArgs a)
     const int y_begin = sy * rows, y_end = min(y_begin + rows, ny);
     const size_t plane = (size_t)ny * pitch;
     const T *src = reinterpret_cast<const T *>(dp->f[a.src]);
-    double col[VEC], acc[5];
+    ObserveSums<VEC> obs;
+    obs.clear();
+    RawVec<ST, VEC> raw[9];
+    auto fetch = [&](int y) {
+        if (valid) {
 #pragma unroll
-    for (int j = 0; j < VEC; ++j) col[j] = 0.0;
-#pragma unroll
-    for (int q = 0; q < 5; ++q) acc[q] = 0.0;
+            for (int i = 0; i < 9; ++i) raw[i] = load_raw<ST, VEC>(src + i * plane + (size_t)y * pitch + x0);
+        }
+    };
+    fetch(y_begin);
     for (int y = y_begin; y < y_end; ++y) {
         float g[9][VEC];
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
             if (valid) {
-                load_vec<ST, VEC>(src + i * plane + (size_t)y * pitch + x0, sh.q9(i), g[i]);
+                expand_raw<ST, VEC>(raw[i], sh.q9(i), g[i]);
             } else {
 #pragma unroll
                 for (int j = 0; j < VEC; ++j) g[i][j] = 0.f;
             }
         }
-        observe_row<VEC>(g, valid, col, acc, dp->rowp + (size_t)sx * ny + y, lane);
+        fetch(min(y + 1, y_end - 1));  // in flight during this row's sums and shuffles
+        observe_row<VEC>(g, valid, obs, dp->rowp + (size_t)sx * ny + y, lane);
     }
-    observe_flush<VEC>(dp->colp, dp->scal, nx, s, sy, x0, valid, col, acc, lane);
+    observe_flush<VEC>(dp->colp, dp->scal, nx, s, sy, x0, valid, obs, lane);
 }
 
 }  // namespace lbm

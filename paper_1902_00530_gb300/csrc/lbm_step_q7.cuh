@@ -230,7 +230,7 @@ __device__ __forceinline__ void noise_u7(uint32_t x, uint32_t y, uint32_t t, uin
 }
 
 template <int VEC>
-__device__ __forceinline__ void observe_row7(const float g[7][VEC], bool valid, double col[VEC], double acc[5],
+__device__ __forceinline__ void observe_row7(const float g[7][VEC], bool valid, ObserveSums<VEC> &o,
                                              double *row_out, int lane)
 {
     float rv[VEC], jxv[VEC], jyv[VEC];
@@ -240,7 +240,7 @@ __device__ __forceinline__ void observe_row7(const float g[7][VEC], bool valid, 
         jxv[j] = (g[1][j] - g[4][j]) + 0.5f * ((g[2][j] + g[6][j]) - (g[3][j] + g[5][j]));
         jyv[j] = Q7_HALF_SQRT3 * ((g[2][j] + g[3][j]) - (g[5][j] + g[6][j]));
     }
-    observe_moments<VEC>(rv, jxv, jyv, valid, col, acc, row_out, lane);
+    observe_moments<VEC>(rv, jxv, jyv, valid, o, row_out, lane);
 }
 
 // Per-warp state of the row walk.
@@ -248,7 +248,7 @@ template <int VEC>
 struct Q7Walk {
     float fc[7][VEC];                     // populations of the current row (MIPS: pulled one row ahead)
     float rm[VEC + 2], rc[VEC + 2], rn[VEC + 2];
-    double col[VEC], acc[5];
+    ObserveSums<VEC> obs;
 };
 
 template <int MODEL, int ST, int VEC, bool SAMPLE, int P>
@@ -295,7 +295,7 @@ __device__ __forceinline__ void q7_row(Q7Walk<VEC> &w, int y, const typename Sto
 #pragma unroll
             for (int j = 0; j < VEC; ++j)
                 g[i][j] = Store<ST>::get(Store<ST>::put(out[i][j], sh.q7(i)), sh.q7(i));
-        observe_row7<VEC>(g, valid, w.col, w.acc, rowp + y, lane);
+        observe_row7<VEC>(g, valid, w.obs, rowp + y, lane);
     }
     if constexpr (MODEL == MODEL_MIPS) {
 #pragma unroll
@@ -336,12 +336,7 @@ __device__ __forceinline__ void direct_strip_q7(const StepArgs &a, const LatDesc
     double *rowp = dp->rowp + (size_t)sx * ny;
 
     Q7Walk<VEC> w;
-    if constexpr (SAMPLE) {
-#pragma unroll
-        for (int j = 0; j < VEC; ++j) w.col[j] = 0.0;
-#pragma unroll
-        for (int q = 0; q < 5; ++q) w.acc[q] = 0.0;
-    }
+    if constexpr (SAMPLE) w.obs.clear();
     if constexpr (MODEL == MODEL_MIPS) {
         float tmp[7][VEC];
         const int yp = wrap_once(y_begin - 1, ny);  // odd
@@ -356,7 +351,7 @@ __device__ __forceinline__ void direct_strip_q7(const StepArgs &a, const LatDesc
         q7_row<MODEL, ST, VEC, SAMPLE, 1>(w, y + 1, src, dst, plane, nx, ny, pitch, x0, valid, last, lane, sh, d,
                                           noise, t, id, a.rk, rowp);
     }
-    if constexpr (SAMPLE) observe_flush<VEC>(dp->colp, dp->scal, nx, s, sy, x0, valid, w.col, w.acc, lane);
+    if constexpr (SAMPLE) observe_flush<VEC>(dp->colp, dp->scal, nx, s, sy, x0, valid, w.obs, lane);
 }
 
 template <int MODEL, int ST, int VEC, bool SAMPLE, int NOISE>
@@ -405,25 +400,31 @@ __global__ void __launch_bounds__(256) observe_kernel_q7(const StepArgs a)
     const int y_begin = sy * rows, y_end = min(y_begin + rows, ny);
     const size_t plane = (size_t)ny * pitch;
     const T *src = reinterpret_cast<const T *>(dp->f[a.src]);
-    double col[VEC], acc[5];
+    ObserveSums<VEC> obs;
+    obs.clear();
+    RawVec<ST, VEC> raw[7];
+    auto fetch = [&](int y) {
+        if (valid) {
 #pragma unroll
-    for (int j = 0; j < VEC; ++j) col[j] = 0.0;
-#pragma unroll
-    for (int q = 0; q < 5; ++q) acc[q] = 0.0;
+            for (int i = 0; i < 7; ++i) raw[i] = load_raw<ST, VEC>(src + i * plane + (size_t)y * pitch + x0);
+        }
+    };
+    fetch(y_begin);
     for (int y = y_begin; y < y_end; ++y) {
         float g[7][VEC];
 #pragma unroll
         for (int i = 0; i < 7; ++i) {
             if (valid) {
-                load_vec<ST, VEC>(src + i * plane + (size_t)y * pitch + x0, sh.q7(i), g[i]);
+                expand_raw<ST, VEC>(raw[i], sh.q7(i), g[i]);
             } else {
 #pragma unroll
                 for (int j = 0; j < VEC; ++j) g[i][j] = 0.f;
             }
         }
-        observe_row7<VEC>(g, valid, col, acc, dp->rowp + (size_t)sx * ny + y, lane);
+        fetch(min(y + 1, y_end - 1));  // in flight during this row's sums and shuffles
+        observe_row7<VEC>(g, valid, obs, dp->rowp + (size_t)sx * ny + y, lane);
     }
-    observe_flush<VEC>(dp->colp, dp->scal, nx, s, sy, x0, valid, col, acc, lane);
+    observe_flush<VEC>(dp->colp, dp->scal, nx, s, sy, x0, valid, obs, lane);
 }
 
 }  // namespace lbm

@@ -240,13 +240,8 @@ __global__ void __maxnreg__(staged_max_regs<VEC>()) step_staged_kernel_q7(const 
         return ok;
     };
 
-    double col[VEC], acc[5];
-    if constexpr (SAMPLE) {
-#pragma unroll
-        for (int j = 0; j < VEC; ++j) col[j] = 0.0;
-#pragma unroll
-        for (int q = 0; q < 5; ++q) acc[q] = 0.0;
-    }
+    ObserveSums<VEC> obs;
+    if constexpr (SAMPLE) obs.clear();
     double *rowp = dp->rowp + (size_t)sx * ny;
 
     float rm[VEC + 2], rc[VEC + 2], rn[VEC + 2];
@@ -316,7 +311,7 @@ __global__ void __maxnreg__(staged_max_regs<VEC>()) step_staged_kernel_q7(const 
 #pragma unroll
                 for (int j = 0; j < VEC; ++j)
                     g[i][j] = Store<ST>::get(Store<ST>::put(out[i][j], sh.q7(i)), sh.q7(i));
-            observe_row7<VEC>(g, valid, col, acc, rowp + y, lane);
+            observe_row7<VEC>(g, valid, obs, rowp + y, lane);
         }
         if constexpr (MIPS) {
 #pragma unroll
@@ -339,7 +334,7 @@ __global__ void __maxnreg__(staged_max_regs<VEC>()) step_staged_kernel_q7(const 
             (void)stage_wait(&full[qq % S], (uint32_t)((qq / S) & 1));
     }
     if (!ok) return;
-    if constexpr (SAMPLE) observe_flush<VEC>(dp->colp, dp->scal, nx, s, sy, x0, valid, col, acc, lane);
+    if constexpr (SAMPLE) observe_flush<VEC>(dp->colp, dp->scal, nx, s, sy, x0, valid, obs, lane);
 }
 
 template <int MODEL, int ST, int VEC, bool SAMPLE, int NOISE>

@@ -400,13 +400,8 @@ __global__ void __maxnreg__(staged_max_regs<VEC>()) step_staged_kernel(const Ste
         return ok;
     };
 
-    double col[VEC], acc[5];
-    if constexpr (SAMPLE) {
-#pragma unroll
-        for (int j = 0; j < VEC; ++j) col[j] = 0.0;
-#pragma unroll
-        for (int q = 0; q < 5; ++q) acc[q] = 0.0;
-    }
+    ObserveSums<VEC> obs;
+    if constexpr (SAMPLE) obs.clear();
 
     // MIPS: row q+1's densities are taken one row ahead of its update.  With
     // CONV its pulled populations are converted then too, into converted row
@@ -473,7 +468,7 @@ __global__ void __maxnreg__(staged_max_regs<VEC>()) step_staged_kernel(const Ste
 #pragma unroll
                 for (int j = 0; j < VEC; ++j)
                     g[i][j] = Store<ST>::get(Store<ST>::put(out[i][j], sh.q9(i)), sh.q9(i));
-            observe_row<VEC>(g, valid, col, acc, dp->rowp + (size_t)sx * ny + y, lane);
+            observe_row<VEC>(g, valid, obs, dp->rowp + (size_t)sx * ny + y, lane);
         }
         if constexpr (MIPS) {
 #pragma unroll
@@ -491,7 +486,7 @@ __global__ void __maxnreg__(staged_max_regs<VEC>()) step_staged_kernel(const Ste
             (void)stage_wait(&full[qq % S], (uint32_t)((qq / S) & 1));
     }
     if (!ok) return;
-    if constexpr (SAMPLE) observe_flush<VEC>(dp->colp, dp->scal, nx, s, sy, x0, valid, col, acc, lane);
+    if constexpr (SAMPLE) observe_flush<VEC>(dp->colp, dp->scal, nx, s, sy, x0, valid, obs, lane);
 }
 
 
