@@ -752,6 +752,15 @@ lbm_status ensure_pinned(lbm_ctx *c)
     return LBM_OK;
 }
 
+// 16-bit populations cross to and from the host as FP32 that the device
+// converts (a host core takes 1 ns and more per value).  They are staged in the
+// lattice's spare buffer, whose content no call reads: how many FP32 planes
+// it holds (Q planes of 16-bit values: at least Q / 2).
+int staging_planes(const LatHost &L)
+{
+    return (int)std::min<size_t>(L.q, L.buf_bytes / ((size_t)L.lat.nx * L.lat.ny * sizeof(float)));
+}
+
 lbm_status require_ready(lbm_ctx *c, bool need_init)
 {
     if (!c) return LBM_ERR_INVALID_ARG;
@@ -1289,8 +1298,7 @@ lbm_status lbm_moments(lbm_ctx *c, int32_t lattice, float *rho, float *ux, float
     if (lattice < 0 || lattice >= (int32_t)c->lats.size()) return fail(c, LBM_ERR_INVALID_ARG, "bad lattice index");
     if (!rho || !ux || !uy) return fail(c, LBM_ERR_INVALID_ARG, "null output pointer");
     const LatHost &L = c->lats[lattice];
-    CK(launch_moments(L.lat.storage, all_desc(c), lattice, (long long)L.lat.nx * L.lat.ny, c->parity, rho, ux,
-                      uy, c->stream),
+    CK(launch_moments(L.lat.storage, all_desc(c), lattice, L.q, L.lat.nx, L.lat.ny, c->parity, rho, ux, uy, c->stream),
        "launch moments kernel");
     return LBM_OK;
 }
@@ -1367,36 +1375,25 @@ lbm_status lbm_get_state(lbm_ctx *c, int32_t lattice, float *dst, int32_t dst_is
     if (lattice < 0 || lattice >= (int32_t)c->lats.size() || !dst)
         return fail(c, LBM_ERR_INVALID_ARG, "bad lattice index or null output");
     const LatHost &L = c->lats[lattice];
-    const char *src = c->state + L.state_off + (c->parity ? L.buf_bytes : 0);
-    const size_t eb = elem_bytes(L.lat.storage);
-    const long long cells = (long long)L.lat.nx * L.lat.ny;
-    if (L.lat.storage == LBM_F32) {
-        CK(cudaMemcpy2DAsync(dst, L.lat.nx * 4, src, L.pitch * 4, L.lat.nx * 4, (size_t)L.q * L.lat.ny,
-                             dst_is_host ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice, c->stream),
+    const int nx = L.lat.nx, ny = L.lat.ny;
+    if (!dst_is_host) {
+        CK(launch_export(L.lat.storage, all_desc(c), lattice, 0, L.q, nx, ny, c->parity, dst, c->stream),
+           "launch export");
+    } else if (L.lat.storage == LBM_F32) {
+        const char *src = c->state + L.state_off + (c->parity ? L.buf_bytes : 0);
+        CK(cudaMemcpy2DAsync(dst, nx * 4, src, L.pitch * 4, nx * 4, (size_t)L.q * ny, cudaMemcpyDeviceToHost, c->stream),
            "copy populations");
-    } else if (!dst_is_host) {
-        CK(launch_export(L.lat.storage, all_desc(c), lattice, cells, c->parity, dst, c->stream), "launch export");
     } else {
-        std::vector<uint16_t> raw((size_t)L.q * cells);
-        CK(cudaMemcpy2DAsync(raw.data(), L.lat.nx * eb, src, L.pitch * eb, L.lat.nx * eb, (size_t)L.q * L.lat.ny,
-                             cudaMemcpyDeviceToHost, c->stream),
-           "copy populations");
-        CK(cudaStreamSynchronize(c->stream), "synchronise");
-        for (int i = 0; i < L.q; ++i) {
-            const float shift = host_shift(L).of(L.q, i);
-            for (long long q = 0; q < cells; ++q) {
-                const uint16_t bits = raw[(size_t)i * cells + q];
-                float v;
-                if (L.lat.storage == LBM_F16_SHIFTED) {
-                    __half h;
-                    std::memcpy(&h, &bits, 2);
-                    v = __half2float(h);
-                } else {
-                    const uint32_t w = (uint32_t)bits << 16;
-                    std::memcpy(&v, &w, 4);
-                }
-                dst[(size_t)i * cells + q] = v + shift;
-            }
+        // expanded on the device, as many populations at a time as the spare buffer holds
+        const int most = staging_planes(L);
+        float *const stage = reinterpret_cast<float *>(c->state + L.state_off + (c->parity ? 0 : L.buf_bytes));
+        const size_t plane = (size_t)nx * ny;
+        for (int i = 0; i < L.q; i += most) {
+            const int np = std::min(most, L.q - i);
+            CK(launch_export(L.lat.storage, all_desc(c), lattice, i, np, nx, ny, c->parity, stage, c->stream),
+               "launch export");
+            CK(cudaMemcpyAsync(dst + i * plane, stage, np * plane * sizeof(float), cudaMemcpyDeviceToHost, c->stream),
+               "copy populations");
         }
     }
     CK(cudaStreamSynchronize(c->stream), "synchronise");
@@ -1416,35 +1413,25 @@ lbm_status lbm_set_state(lbm_ctx *c, int32_t lattice, const float *src, int32_t 
         c->initialized = true;
     }
     const LatHost &L = c->lats[lattice];
-    char *dstp = c->state + L.state_off + (c->parity ? L.buf_bytes : 0);
-    const size_t eb = elem_bytes(L.lat.storage);
-    const long long cells = (long long)L.lat.nx * L.lat.ny;
-    if (L.lat.storage == LBM_F32) {
-        CK(cudaMemcpy2DAsync(dstp, L.pitch * 4, src, L.lat.nx * 4, L.lat.nx * 4, (size_t)L.q * L.lat.ny,
-                             src_is_host ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, c->stream),
+    const int nx = L.lat.nx, ny = L.lat.ny;
+    if (!src_is_host) {
+        CK(launch_import(L.lat.storage, all_desc(c), lattice, 0, L.q, nx, ny, c->parity, src, c->stream),
+           "launch import");
+    } else if (L.lat.storage == LBM_F32) {
+        char *dstp = c->state + L.state_off + (c->parity ? L.buf_bytes : 0);
+        CK(cudaMemcpy2DAsync(dstp, L.pitch * 4, src, nx * 4, nx * 4, (size_t)L.q * ny, cudaMemcpyHostToDevice, c->stream),
            "copy populations");
-    } else if (!src_is_host) {
-        CK(launch_import(L.lat.storage, all_desc(c), lattice, cells, c->parity, src, c->stream), "launch import");
     } else {
-        std::vector<uint16_t> raw((size_t)L.q * cells);
-        for (int i = 0; i < L.q; ++i) {
-            const float shift = host_shift(L).of(L.q, i);
-            for (long long q = 0; q < cells; ++q) {
-                const float v = src[(size_t)i * cells + q] - shift;
-                uint16_t bits;
-                if (L.lat.storage == LBM_F16_SHIFTED) {
-                    const __half h = __float2half_rn(v);
-                    std::memcpy(&bits, &h, 2);
-                } else {
-                    const __nv_bfloat16 b = __float2bfloat16_rn(v);
-                    std::memcpy(&bits, &b, 2);
-                }
-                raw[(size_t)i * cells + q] = bits;
-            }
+        const int most = staging_planes(L);
+        float *const stage = reinterpret_cast<float *>(c->state + L.state_off + (c->parity ? 0 : L.buf_bytes));
+        const size_t plane = (size_t)nx * ny;
+        for (int i = 0; i < L.q; i += most) {
+            const int np = std::min(most, L.q - i);
+            CK(cudaMemcpyAsync(stage, src + i * plane, np * plane * sizeof(float), cudaMemcpyHostToDevice, c->stream),
+               "copy populations");
+            CK(launch_import(L.lat.storage, all_desc(c), lattice, i, np, nx, ny, c->parity, stage, c->stream),
+               "launch import");
         }
-        CK(cudaMemcpy2DAsync(dstp, L.pitch * eb, raw.data(), L.lat.nx * eb, L.lat.nx * eb, (size_t)L.q * L.lat.ny,
-                             cudaMemcpyHostToDevice, c->stream),
-           "copy populations");
     }
     CK(cudaStreamSynchronize(c->stream), "synchronise");
     return LBM_OK;
@@ -1459,7 +1446,7 @@ lbm_status lbm_add_density(lbm_ctx *c, int32_t lattice, double delta_rho_bar)
     for (int k = 0; k < (int)c->lats.size(); ++k) {
         if (lattice != -1 && k != lattice) continue;
         const LatHost &L = c->lats[k];
-        CK(launch_add_density(L.lat.storage, all_desc(c), k, (long long)L.lat.nx * L.lat.ny, c->parity,
+        CK(launch_add_density(L.lat.storage, all_desc(c), k, L.q, L.lat.nx, L.lat.ny, c->parity,
                               (float)(delta_rho_bar / (double)L.q), c->stream),
            "launch density step");
     }

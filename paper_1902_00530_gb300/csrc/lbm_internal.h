@@ -53,23 +53,23 @@ cudaError_t launch_observe_q7_f32(int vec, const StepArgs &a, int blocks, int wa
 cudaError_t launch_observe_q7_f16(int vec, const StepArgs &a, int blocks, int warps, cudaStream_t stream);
 cudaError_t launch_observe_q7_bf16(int vec, const StepArgs &a, int blocks, int warps, cudaStream_t stream);
 
-// auxiliary kernels (lbm_aux.cu); the lattice's q comes from its descriptor,
-// so `cells` counts sites and q * cells elements are touched
+// auxiliary kernels (lbm_aux.cu)
 size_t init_spec_bytes();
 void pack_init_spec(void *dst, double rho_mean, double rho_amp, int u_kind, double u_amp, double ux0,
                     double uy0, double A, double B);
 cudaError_t launch_init(int storage, const LatDesc *desc, const void *specs, int nlat, long long max_cells,
                         int dst, uint64_t seed, cudaStream_t s);
-cudaError_t launch_moments(int storage, const LatDesc *desc, int lat, long long cells, int src, float *rho,
+cudaError_t launch_moments(int storage, const LatDesc *desc, int lat, int q, int nx, int ny, int src, float *rho,
                            float *ux, float *uy, cudaStream_t s);
-cudaError_t launch_export(int storage, const LatDesc *desc, int lat, long long cells, int src, float *out,
-                          cudaStream_t s);
-cudaError_t launch_import(int storage, const LatDesc *desc, int lat, long long cells, int dst,
+// populations i0 .. i0 + planes - 1 of a lattice to / from dense FP32 [planes][ny][nx]
+cudaError_t launch_export(int storage, const LatDesc *desc, int lat, int i0, int planes, int nx, int ny, int src,
+                          float *out, cudaStream_t s);
+cudaError_t launch_import(int storage, const LatDesc *desc, int lat, int i0, int planes, int nx, int ny, int dst,
                           const float *in, cudaStream_t s);
 cudaError_t launch_finalize(const LatDesc *desc, int nlat, int max_chunk, const uint32_t *t_ptr, uint32_t k,
                             int to_ring, unsigned *err, int want, double *host, cudaStream_t s);
 cudaError_t launch_advance_time(uint32_t *t_ptr, uint32_t n, cudaStream_t s);
-cudaError_t launch_add_density(int storage, const LatDesc *desc, int lat, long long cells, int buf, float per_pop,
+cudaError_t launch_add_density(int storage, const LatDesc *desc, int lat, int q, int nx, int ny, int buf, float per_pop,
                                cudaStream_t s);
 cudaError_t launch_set_time(uint32_t *t_ptr, uint32_t t, cudaStream_t s);
 cudaError_t launch_wait_timeout(unsigned *err, cudaStream_t s);
