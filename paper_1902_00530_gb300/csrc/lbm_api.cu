@@ -43,6 +43,10 @@ constexpr int TUNE_STEPS_MAX = 256;
 // persistent against 29.0 per step, while the tuner's timing form preferred
 // it; 256 of 128^2 (4.2 M): 82.6 against 64.2.
 constexpr long long PERSIST_AUTO_MIN_SITES = 1LL << 20;
+// Groups of at most this many sites per step also try strips of fewer than 8
+// rows: beyond it, 8-row strips of the widest vectors already give every warp
+// slot of the GPU a strip (2^22 sites: 4096 strips of 8 x 128 for 3648 slots).
+constexpr long long SHORT_STRIP_MAX_SITES = 1LL << 22;
 
 size_t align256(size_t v) { return (v + 255) & ~size_t(255); }
 int ceil_div(long long a, long long b) { return (int)((a + b - 1) / b); }
@@ -63,6 +67,10 @@ struct LatHost {
     int64_t consumed = 0;
 };
 
+struct Shape {
+    int vec, rows, warps, stages;
+};
+
 struct GroupHost {
     int model = 0, storage = 0, q = 9;
     std::vector<int> members;
@@ -79,6 +87,11 @@ struct GroupHost {
     bool resident = false;
     int res_cluster = 0, res_threads = 0;
     size_t res_smem = 0;
+    // the tuner's direct shape of short strips for steps that take no sample
+    // (rows = 0: none, they run in the shape above), and its descriptor table
+    Shape plain{0, 0, 0, 0};
+    int plain_blocks = 0;
+    size_t plain_off = 0;
 };
 
 struct GraphKey {
@@ -265,6 +278,8 @@ void layout(lbm_ctx *c)
     for (auto &g : c->groups) {
         g.desc_off = o;
         o = align256(o + g.members.size() * sizeof(LatDesc));
+        g.plain_off = o;
+        o = align256(o + g.members.size() * sizeof(LatDesc));
     }
     for (auto &g : c->groups) {
         // the work counter in a slot of its own, then the progress counters of
@@ -315,7 +330,7 @@ Shift3 host_shift(const LatHost &L)
     return s;
 }
 
-LatDesc make_desc(const lbm_ctx *c, const LatHost &L, int block_begin, const GroupHost &g)
+LatDesc make_desc(const lbm_ctx *c, const LatHost &L, int block_begin, const Shape &g)
 {
     LatDesc d;
     std::memset(&d, 0, sizeof(d));
@@ -374,7 +389,7 @@ lbm_status upload_descs(lbm_ctx *c)
         int blocks = 0;
         for (int m : g.members) {
             LatHost &L = c->lats[m];
-            LatDesc d = make_desc(c, L, blocks, g);
+            LatDesc d = make_desc(c, L, blocks, {g.vec, g.rows, g.warps, g.stages});
             L.nsx = d.nsx;
             L.nsy = d.nsy;
             L.nchunk = d.nchunk;
@@ -393,6 +408,17 @@ lbm_status upload_descs(lbm_ctx *c)
         CK(cudaMemcpyAsync(c->scratch + g.desc_off, gd.data(), gd.size() * sizeof(LatDesc),
                            cudaMemcpyHostToDevice, c->stream),
            "upload group descriptors");
+        if (g.plain.rows > 0) {
+            gd.clear();
+            g.plain_blocks = 0;
+            for (int m : g.members) {
+                gd.push_back(make_desc(c, c->lats[m], g.plain_blocks, g.plain));
+                g.plain_blocks += ceil_div((long long)gd.back().nsx * gd.back().nsy, g.plain.warps);
+            }
+            CK(cudaMemcpyAsync(c->scratch + g.plain_off, gd.data(), gd.size() * sizeof(LatDesc),
+                               cudaMemcpyHostToDevice, c->stream),
+               "upload short-strip descriptors");
+        }
         // lattice groups of the persistent launch: consecutive members whose
         // two population buffers each fit the L2 budget together (at least one
         // lattice per group); entry i is the group's first block of the step grid
@@ -458,21 +484,27 @@ int group_noise(const lbm_ctx *c, const GroupHost &g)
 cudaError_t launch_group_step(const lbm_ctx *c, const GroupHost &g, int src, uint32_t k, bool sample,
                               cudaStream_t stream)
 {
-    const StepArgs a = step_args(c, g, src, k);
+    StepArgs a = step_args(c, g, src, k);
     const int noise = group_noise(c, g);
-    const int kind = g.stages > 0 ? 1 : 0;
+    int kind = g.stages > 0 ? 1 : 0, vec = g.vec, blocks = g.blocks, warps = g.warps;
+    if (!sample && g.plain.rows > 0) {
+        a.desc = reinterpret_cast<const LatDesc *>(c->scratch + g.plain_off);
+        a.stages = kind = 0;
+        vec = g.plain.vec;
+        blocks = g.plain_blocks;
+        warps = g.plain.warps;
+    }
     if (g.q == 7) {
         if (g.storage == LBM_F32)
-            return launch_step_q7_f32(g.model, kind, g.vec, sample, noise, a, g.blocks, g.warps, stream);
+            return launch_step_q7_f32(g.model, kind, vec, sample, noise, a, blocks, warps, stream);
         if (g.storage == LBM_F16_SHIFTED)
-            return launch_step_q7_f16(g.model, kind, g.vec, sample, noise, a, g.blocks, g.warps, stream);
-        return launch_step_q7_bf16(g.model, kind, g.vec, sample, noise, a, g.blocks, g.warps, stream);
+            return launch_step_q7_f16(g.model, kind, vec, sample, noise, a, blocks, warps, stream);
+        return launch_step_q7_bf16(g.model, kind, vec, sample, noise, a, blocks, warps, stream);
     }
-    if (g.storage == LBM_F32)
-        return launch_step_f32(g.model, kind, g.vec, sample, noise, a, g.blocks, g.warps, stream);
+    if (g.storage == LBM_F32) return launch_step_f32(g.model, kind, vec, sample, noise, a, blocks, warps, stream);
     if (g.storage == LBM_F16_SHIFTED)
-        return launch_step_f16(g.model, kind, g.vec, sample, noise, a, g.blocks, g.warps, stream);
-    return launch_step_bf16(g.model, kind, g.vec, sample, noise, a, g.blocks, g.warps, stream);
+        return launch_step_f16(g.model, kind, vec, sample, noise, a, blocks, warps, stream);
+    return launch_step_bf16(g.model, kind, vec, sample, noise, a, blocks, warps, stream);
 }
 
 // Groups the persistent launch can take: those on a direct kernel (D2Q9 or D2Q7).
@@ -769,10 +801,6 @@ lbm_status require_ready(lbm_ctx *c, bool need_init)
     return LBM_OK;
 }
 
-struct Shape {
-    int vec, rows, warps, stages;
-};
-
 // A pair of timing events, destroyed on every way out of the tuner.
 struct EventPair {
     cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -795,10 +823,24 @@ struct EventPair {
 // form.  With persistent launches on (mode 1) direct candidates are timed as
 // persistent launches; in mode 2 both ways, and the faster way is kept with
 // the shape.
-struct Alt {
+// How a group runs: the shape of its launches, the short strips of plain
+// steps (rows 0: none), and the launch form of stretches of plain steps.
+struct Choice {
     Shape shape;
-    bool persist, resident;
+    Shape plain = {0, 0, 0, 0};
+    bool persist = false, resident = false;
 };
+Choice choice_of(const GroupHost &g) { return {{g.vec, g.rows, g.warps, g.stages}, g.plain, g.persist, g.resident}; }
+void choose(GroupHost &g, const Choice &ch)
+{
+    g.vec = ch.shape.vec;
+    g.rows = ch.shape.rows;
+    g.warps = ch.shape.warps;
+    g.stages = ch.shape.stages;
+    g.plain = ch.plain;
+    g.persist = ch.persist;
+    g.resident = ch.resident;
+}
 
 // The resident launch's plan for a group: the cluster size (blocks per
 // lattice) with the least estimated time per step, if any fits.  A step takes
@@ -853,7 +895,7 @@ bool plan_resident(const lbm_ctx *c, GroupHost &g)
     return best < 1e29;
 }
 
-lbm_status tune_group(lbm_ctx *c, GroupHost &g, std::vector<Alt> *alts)
+lbm_status tune_group(lbm_ctx *c, GroupHost &g, std::vector<Choice> *alts)
 {
     std::vector<Shape> cands;
     long long max_ny = 1, group_sites = 0;
@@ -893,8 +935,7 @@ lbm_status tune_group(lbm_ctx *c, GroupHost &g, std::vector<Alt> *alts)
     CK(ev.create(), "create event");
     cudaEvent_t e0 = ev.e0, e1 = ev.e1;
     float best = 1e30f, best_kind[2] = {1e30f, 1e30f}, best_step = 1e30f;
-    Shape bs{g.vec, g.rows, g.warps, g.stages}, bk[2] = {bs, bs}, bstep = bs;
-    bool bp = g.persist, bkp[2] = {bp, bp};
+    Choice b = choice_of(g), bk[2] = {b, b}, bstep = b;
     // The time of `steps` steps in the group's current shape and form, scaled
     // to TUNE_STEPS (steps grow until the timing is long enough).
     auto time_form = [&](int steps, float *out) -> lbm_status {
@@ -911,12 +952,8 @@ lbm_status tune_group(lbm_ctx *c, GroupHost &g, std::vector<Alt> *alts)
         *out = ms * (float)TUNE_STEPS / (float)steps;
         return LBM_OK;
     };
-    g.resident = false;
     for (const Shape &sh : cands) {
-        g.vec = sh.vec;
-        g.rows = sh.rows;
-        g.warps = sh.warps;
-        g.stages = sh.stages;
+        choose(g, {sh});
         lbm_status st = upload_descs(c);
         if (st != LBM_OK) return st;
         // launch forms to time: as lbm_step would launch it (modes 0, 1), or
@@ -933,68 +970,78 @@ lbm_status tune_group(lbm_ctx *c, GroupHost &g, std::vector<Alt> *alts)
             float ms = 0.f;
             st = time_form(persistent_ok(c, g) ? TUNE_STEPS_PERSIST : TUNE_STEPS, &ms);
             if (st != LBM_OK) return st;
+            const Choice now = choice_of(g);
             if (ms < best) {
                 best = ms;
-                bs = sh;
-                bp = g.persist;
+                b = now;
             }
             const int kind = sh.stages > 0 ? 1 : 0;
             if (ms < best_kind[kind]) {
                 best_kind[kind] = ms;
-                bk[kind] = sh;
-                bkp[kind] = g.persist;
+                bk[kind] = now;
             }
             if (!persistent_ok(c, g) && ms < best_step) {
                 best_step = ms;
-                bstep = sh;
+                bstep = now;
             }
         }
     }
-    const int other = bs.stages > 0 ? 0 : 1;
+    const int other = b.shape.stages > 0 ? 0 : 1;
     alts->clear();
-    if (best_kind[other] < 1e29f) alts->push_back({bk[other], bkp[other], false});
+    if (best_kind[other] < 1e29f) alts->push_back(bk[other]);
     // mode 2, a persistent choice: its best per-step direct form too (beside
     // other groups, a persistent launch holds the SMs its grid fills; the best
     // staged form is the alternative above)
-    if (bp && best_step < 1e29f && bstep.stages == 0) alts->push_back({bstep, false, false});
-    // mode 2: the resident launch where the lattices fit on chip and it is
-    // faster than the best of the others; single and sample steps then take the
-    // best per-step shape
-    bool res = false;
-    g.persist = false;
-    if (c->persist_mode == 2 && best_step < 1e29f && plan_resident(c, g)) {
-        g.resident = true;
-        float ms = 0.f;
-        lbm_status st = LBM_OK;
-        if (launch_group_timed(c, g, 1, c->stream) == cudaSuccess)
-            st = time_form(TUNE_STEPS_PERSIST, &ms);
-        else
-            cudaGetLastError(), ms = 1e30f;
+    if (b.persist && best_step < 1e29f && bstep.shape.stages == 0) alts->push_back(bstep);
+    // `now`, built on the best per-step shape (which single and sample steps
+    // keep), is chosen where it runs and is the fastest so far
+    auto consider = [&](const Choice &now, int steps) -> lbm_status {
+        choose(g, now);
+        lbm_status st = upload_descs(c);
         if (st != LBM_OK) return st;
-        res = ms < best;
+        if (launch_group_timed(c, g, 1, c->stream) != cudaSuccess) {
+            cudaGetLastError();
+            return LBM_OK;
+        }
+        float ms = 0.f;
+        st = time_form(steps, &ms);
+        if (st != LBM_OK || ms >= best) return st;
+        best = ms;
+        b = now;
+        return LBM_OK;
+    };
+    lbm_status st = LBM_OK;
+    // Strips of fewer than 8 rows, for steps without a sample (which size the
+    // scratch).  A warp walks its rows one after the other, so in a lattice whose
+    // 8-row strips leave warps of the GPU idle a step lasts as long as one
+    // walk; measured (FP32): 720 x 240 D2Q7 CIL 8.7 us per step in 8-row strips.
+    if (c->persist_mode != 1 && best_step < 1e29f && direct && group_sites <= SHORT_STRIP_MAX_SITES)
+        for (int v : {1, 2, 4}) {
+            bool ok = allowed_vec(g.storage, v);
+            for (int m : g.members) ok = ok && (c->lats[m].lat.nx % v == 0);
+            for (int r : {1, 2, 4})
+                for (int w : {4, 8}) {
+                    if (!ok || (g.q == 7 && r == 1)) continue;
+                    Choice now = bstep;
+                    now.plain = {v, r, w, 0};
+                    st = consider(now, TUNE_STEPS);
+                    if (st != LBM_OK) return st;
+                }
+        }
+    if (b.plain.rows > 0) alts->push_back(bstep);
+    // mode 2: the resident launch where the lattices fit on chip
+    if (c->persist_mode == 2 && best_step < 1e29f && plan_resident(c, g)) {
+        const Choice before = b;
+        Choice now = b.persist ? bstep : b;
+        now.resident = true;
+        st = consider(now, TUNE_STEPS_PERSIST);
+        if (st != LBM_OK) return st;
+        if (b.resident) alts->push_back(before);
     }
-    if (res) {
-        alts->push_back({bs, bp, false});
-        bs = bstep;
-        bp = false;
-    }
-    g.resident = res;
-    g.vec = bs.vec;
-    g.rows = bs.rows;
-    g.warps = bs.warps;
-    g.stages = bs.stages;
-    g.persist = bp;
-    lbm_status st = upload_descs(c);
+    choose(g, b);
+    st = upload_descs(c);
     if (st != LBM_OK) return st;
     return read_error_flag(c);
-}
-
-void set_shape(GroupHost &g, const Shape &sh)
-{
-    g.vec = sh.vec;
-    g.rows = sh.rows;
-    g.warps = sh.warps;
-    g.stages = sh.stages;
 }
 
 // TUNE_STEPS_PERSIST steps of every group as lbm_step runs a batch (forked,
@@ -1040,7 +1087,7 @@ lbm_status time_joint_step(lbm_ctx *c, float *ms)
 lbm_status do_tune(lbm_ctx *c)
 {
     const size_t ng = c->groups.size();
-    std::vector<std::vector<Alt>> alts(ng);
+    std::vector<std::vector<Choice>> alts(ng);
     for (size_t gi = 0; gi < ng; ++gi) {
         lbm_status st = tune_group(c, c->groups[gi], &alts[gi]);
         if (st != LBM_OK) return st;
@@ -1053,22 +1100,14 @@ lbm_status do_tune(lbm_ctx *c)
         if (st != LBM_OK) return st;
         for (size_t gi = 0; gi < ng; ++gi) {
             GroupHost &g = c->groups[gi];
-            for (const Alt &al : alts[gi]) {
-                const Shape keep{g.vec, g.rows, g.warps, g.stages};
-                const bool keep_persist = g.persist, keep_resident = g.resident;
-                set_shape(g, al.shape);
-                g.persist = al.persist;
-                g.resident = al.resident;
+            for (const Choice &al : alts[gi]) {
+                const Choice keep = choice_of(g);
+                choose(g, al);
                 float ms = 0.f;
                 st = time_joint_step(c, &ms);
                 if (st != LBM_OK) return st;
-                if (ms < best) {
-                    best = ms;
-                } else {
-                    set_shape(g, keep);
-                    g.persist = keep_persist;
-                    g.resident = keep_resident;
-                }
+                if (ms < best) best = ms;
+                else choose(g, keep);
             }
         }
         st = upload_descs(c);
@@ -1609,6 +1648,7 @@ lbm_status lbm_set_tuning(lbm_ctx *c, int32_t mode, int32_t vec, int32_t rows, i
         g.warps = warps;
         g.stages = stages;
         g.resident = false;
+        g.plain.rows = 0;
     }
     c->tune_mode = 1;
     c->tuned = true;

@@ -289,6 +289,8 @@ __global__ void __launch_bounds__(FIN_THREADS) finalize_kernel(const LatDesc *de
 {
     __shared__ double part[FIN_WARPS][32], S[9];
     __shared__ bool am_last;
+    wait_for_previous();
+    allow_dependents();
     const int l = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (l >= nlat) return;
     const LatDesc *dp = desc + l;
@@ -409,7 +411,11 @@ __global__ void __launch_bounds__(FIN_THREADS) finalize_kernel(const LatDesc *de
     __threadfence_system();
 }
 
-__global__ void advance_time_kernel(uint32_t *t_ptr, uint32_t n) { *t_ptr += n; }
+__global__ void advance_time_kernel(uint32_t *t_ptr, uint32_t n)
+{
+    wait_for_previous();
+    *t_ptr += n;
+}
 
 __global__ void set_time_kernel(uint32_t *t_ptr, uint32_t t) { *t_ptr = t; }
 
@@ -564,14 +570,12 @@ cudaError_t launch_finalize(const LatDesc *desc, int nlat, int max_chunk, const 
                             int to_ring, unsigned *err, int want, double *host, cudaStream_t s)
 {
     dim3 g(max_chunk, nlat);
-    finalize_kernel<<<g, FIN_THREADS, 0, s>>>(desc, nlat, t_ptr, k, to_ring, err, want, host);
-    return cudaGetLastError();
+    return launch_dependent(finalize_kernel, g, dim3(FIN_THREADS), 0, s, desc, nlat, t_ptr, k, to_ring, err, want, host);
 }
 
 cudaError_t launch_advance_time(uint32_t *t_ptr, uint32_t n, cudaStream_t s)
 {
-    advance_time_kernel<<<1, 1, 0, s>>>(t_ptr, n);
-    return cudaGetLastError();
+    return launch_dependent(advance_time_kernel, dim3(1), dim3(1), 0, s, t_ptr, n);
 }
 
 cudaError_t launch_wait_timeout(unsigned *err, cudaStream_t s)

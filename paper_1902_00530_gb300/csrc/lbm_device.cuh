@@ -416,6 +416,35 @@ __device__ __forceinline__ float load_one(const typename Store<ST>::T *p, float 
     return Store<ST>::get(p[0], shift);
 }
 
+// Programmatic dependent launch.  Consecutive steps are dependent launches, and
+// between two plain ones the GPU idles for about a microsecond: the end of the last
+// block, the signal, the next grid's launch.  A kernel launched by
+// launch_dependent may be put on the SMs while the one before it in the stream
+// still runs (from when all of that one's blocks have called
+// allow_dependents); wait_for_previous then holds its blocks until the one before
+// has finished and its stores are visible, so a step still sees whole steps only.
+// Each kernel launched this way calls wait_for_previous before its first access to
+// global memory, also to have the waits of a chain of launches imply one
+// another.
+__device__ __forceinline__ void allow_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <typename Kernel, typename... Args>
+inline cudaError_t launch_dependent(Kernel kern, dim3 grid, dim3 block, size_t smem, cudaStream_t stream, Args... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
 __device__ __forceinline__ int wrap_once(int a, int n)
 {
     a = a < 0 ? a + n : a;

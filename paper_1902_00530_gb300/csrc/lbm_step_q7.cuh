@@ -357,6 +357,8 @@ __device__ __forceinline__ void direct_strip_q7(const StepArgs &a, const LatDesc
 template <int MODEL, int ST, int VEC, bool SAMPLE, int NOISE>
 __global__ void __launch_bounds__(256) step_kernel_q7(const StepArgs a)
 {
+    wait_for_previous();
+    allow_dependents();
     const LatDesc *dp = a.desc + find_lattice(a.desc, a.nlat, blockIdx.x);
     const int s = (blockIdx.x - dp->block_begin) * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (s >= dp->nsx * dp->nsy) return;  // whole warp leaves together

@@ -60,7 +60,7 @@ def _same(storage, cfg, calls=(7, 6), every=0, graphs=True, fits=True):
     b, lb, sb = _run(0, storage, cfg, calls, every, graphs)
     for k, (x, y) in enumerate(zip(a, b)):
         np.testing.assert_array_equal(x, y, err_msg=f"lattice {k}")
-    if fits:
+    if fits and max(n[0] * n[1] for n in cfg) <= SURE:
         assert all(p < q for p, q in zip(la, lb)), (la, lb)  # the stretches ran as one launch each
     if every:
         for x, y in zip(sa, sb):
@@ -69,6 +69,10 @@ def _same(storage, cfg, calls=(7, 6), every=0, graphs=True, fits=True):
 
 
 C2 = W.INIT_CONFIG2
+# sites up to which a lattice that fits runs resident for certain (several times faster than the
+# other forms); beyond, the tuner's timings decide.  [2, 2]: the stretch and the time advance,
+# [8, 7]: its steps and the time advance.
+SURE = 10800
 SIZES9 = [(64, 64), (1, 7), (2, 5), (33, 2), (90, 31), (801, 20), (200, 150)]
 SIZES7 = [(90, 30), (1, 8), (2, 6), (33, 4), (180, 60), (801, 22), (180, 150)]
 
@@ -79,7 +83,7 @@ SIZES7 = [(90, 30), (1, 8), (2, 6), (33, 4), (180, 60), (801, 22), (180, 150)]
 def test_resident_equals_per_step_d2q9(size, preset, storage):
     fits = _fits(9, storage, preset, *size)
     launches = _same(storage, [(*size, preset, {}, C2, "d2q9")], fits=fits)
-    assert launches == ([2, 2] if fits else [8, 7])  # the stretch (or its steps) and the time advance
+    assert launches in ([[2, 2]] if fits and size[0] * size[1] <= SURE else [[2, 2], [8, 7]] if fits else [[8, 7]])
 
 
 @pytest.mark.parametrize("storage", ["f32", "bf16s"])
@@ -88,7 +92,7 @@ def test_resident_equals_per_step_d2q9(size, preset, storage):
 def test_resident_equals_per_step_d2q7(size, preset, storage):
     fits = _fits(7, storage, preset, *size)
     launches = _same(storage, [(*size, preset, {}, C2, "d2q7")], fits=fits)
-    assert launches == ([2, 2] if fits else [8, 7])  # the stretch (or its steps) and the time advance
+    assert launches in ([[2, 2]] if fits and size[0] * size[1] <= SURE else [[2, 2], [8, 7]] if fits else [[8, 7]])
 
 
 @pytest.mark.parametrize("graphs", [True, False])
