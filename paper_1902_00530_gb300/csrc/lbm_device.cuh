@@ -139,6 +139,7 @@ struct StepArgs {
     uint32_t k;           // step offset of this launch from *t_ptr
     uint32_t key0, key1;  // Philox key = seed
     int stages;           // staged kernel: shared-memory row buffers per warp
+    int ragged;           // direct kernel: the vector width need not divide nx
     unsigned *err;        // device error word (bounded waits report here)
     uint32_t rk[20];      // Philox round keys: (key0 + r W0, key1 + r W1), r = 0..9
 };

@@ -126,6 +126,32 @@ __device__ __forceinline__ void pull_row_wide(const typename Store<ST>::T *base,
     pull_pop_wide<ST, VEC, 8>(base + 8 * plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q9(8), f[8]);
 }
 
+// A row whose length is no multiple of VEC ends inside one lane's vector: its
+// first nv = nx - x0 sites are the row's, the others lie in the padding of the
+// pitch (loaded, updated and stored there for nothing; no call reads them).  The
+// pull put the site after them, padding, into the last real site's x + 1
+// populations; this puts the row's first site there.
+template <int ST, int VEC>
+__device__ __forceinline__ void wrap_partial(const typename Store<ST>::T *base, size_t plane, int y, int ny, int pitch,
+                                             int nv, const Shift3 &sh, float f[9][VEC])
+{
+#pragma unroll
+    for (int i = 1; i < 9; ++i) {
+        if (vx(i) != -1) continue;
+        const float v = load_one<ST>(base + i * plane + (size_t)wrap_once(y - vy(i), ny) * pitch, sh.q9(i));
+#pragma unroll
+        for (int j = 0; j < VEC - 1; ++j)
+            if (j == nv - 1) f[i][j] = v;
+    }
+}
+// The same for a row's density window (r[k] is site x0 + k - 1).
+template <int VEC> __device__ __forceinline__ void wrap_partial_window(int nv, float right, float r[VEC + 2])
+{
+#pragma unroll
+    for (int k = 2; k < VEC + 1; ++k)
+        if (k == nv + 1) r[k] = right;
+}
+
 template <int VEC>
 __device__ __forceinline__ float density(const float f[9][VEC], int j)
 {
@@ -141,7 +167,7 @@ __device__ __forceinline__ float density(const float f[9][VEC], int j)
 // one, and a shuffle tree adds them in density()'s order (((f0+f1)+(f2+f3)) +
 // ((f4+f5)+(f6+f7))) + f8, so the sums are bitwise those of a single-lane
 // pull without its nine serial loads.
-template <int ST, int VEC>
+template <int ST, int VEC, bool RAGGED>
 __device__ __forceinline__ void density_window(const float f[9][VEC], const typename Store<ST>::T *base,
                                                uint32_t plane, int y, int nx, int ny, int pitch, int x0,
                                                bool valid, bool last, int lane, const Shift3 &sh,
@@ -169,6 +195,7 @@ __device__ __forceinline__ void density_window(const float f[9][VEC], const type
     if (last) right = halo_right;
     r[0] = left;
     r[VEC + 1] = right;
+    if (RAGGED && valid && x0 + VEC > nx) wrap_partial_window<VEC>(nx - x0, right, r);
 }
 
 // Model parameters of one lattice, held in registers.
@@ -708,8 +735,10 @@ template <int MODEL, int ST, int VEC, bool SAMPLE> constexpr int direct_min_bloc
 
 // One warp's strip s (< nsx nsy) of lattice dp for the step at time t, read
 // from buffer `src` and written to the other: the body of the direct kernel,
-// shared by the per-step launch and the persistent launch.
-template <int MODEL, int ST, int VEC, bool SAMPLE, int NOISE>
+// shared by the per-step launch and the persistent launch.  RAGGED: VEC need not
+// divide nx (see wrap_partial; a form of its own, since the test for it in every
+// row cost the others 5 to 9 %: 1024^2 CIL 14.3 -> 15.1 us, MIPS 21.9 -> 24.6).
+template <int MODEL, int ST, int VEC, bool SAMPLE, int NOISE, bool RAGGED = false>
 __device__ __forceinline__ void direct_strip(const StepArgs &a, const LatDesc *dp, int s, int src_buf, uint32_t t)
 {
     using T = typename Store<ST>::T;
@@ -721,6 +750,7 @@ __device__ __forceinline__ void direct_strip(const StepArgs &a, const LatDesc *d
     const int x0 = sx * 32 * VEC + lane * VEC;
     const bool valid = x0 < nx;
     const bool last = (lane == 31) || (x0 + VEC >= nx);
+    const bool partial = RAGGED && valid && x0 + VEC > nx;
     const int y_begin = sy * rows, y_end = min(y_begin + rows, ny);
     const size_t plane = (size_t)ny * pitch;
     const uint32_t plane32 = (uint32_t)plane;  // q ny pitch <= 2^32 (host check) where used
@@ -745,9 +775,11 @@ __device__ __forceinline__ void direct_strip(const StepArgs &a, const LatDesc *d
         float tmp[9][VEC];
         const int yp = wrap_once(y_begin - 1, ny);
         pull_row<ST, VEC>(src, plane32, yp, ny, nx, pitch, x0, valid, last, lane, sh, tmp);
-        density_window<ST, VEC>(tmp, src, plane32, yp, nx, ny, pitch, x0, valid, last, lane, sh, rm);
+        if (partial) wrap_partial<ST, VEC>(src, plane, yp, ny, pitch, nx - x0, sh, tmp);
+        density_window<ST, VEC, RAGGED>(tmp, src, plane32, yp, nx, ny, pitch, x0, valid, last, lane, sh, rm);
         pull_row<ST, VEC>(src, plane32, y_begin, ny, nx, pitch, x0, valid, last, lane, sh, tmp);
-        density_window<ST, VEC>(tmp, src, plane32, y_begin, nx, ny, pitch, x0, valid, last, lane, sh, rc);
+        if (partial) wrap_partial<ST, VEC>(src, plane, y_begin, ny, pitch, nx - x0, sh, tmp);
+        density_window<ST, VEC, RAGGED>(tmp, src, plane32, y_begin, nx, ny, pitch, x0, valid, last, lane, sh, rc);
     }
 
     for (int y = y_begin; y < y_end; ++y) {
@@ -768,12 +800,14 @@ __device__ __forceinline__ void direct_strip(const StepArgs &a, const LatDesc *d
             float fn[9][VEC];
             const int yn = wrap_once(y + 1, ny);
             pull_row<ST, VEC>(src, plane32, yn, ny, nx, pitch, x0, valid, last, lane, sh, fn);
-            density_window<ST, VEC>(fn, src, plane32, yn, nx, ny, pitch, x0, valid, last, lane, sh, rn);
+            if (partial) wrap_partial<ST, VEC>(src, plane, yn, ny, pitch, nx - x0, sh, fn);
+            density_window<ST, VEC, RAGGED>(fn, src, plane32, yn, nx, ny, pitch, x0, valid, last, lane, sh, rn);
         }
         if constexpr (WIDE)
             pull_row_wide<ST, VEC>(src, plane, y, ny, nx, pitch, x0, valid, last, lane, sh, fc);
         else
             pull_row<ST, VEC>(src, plane32, y, ny, nx, pitch, x0, valid, last, lane, sh, fc);
+        if (partial) wrap_partial<ST, VEC>(src, plane, y, ny, pitch, nx - x0, sh, fc);
         float gx[VEC], gy[VEC];
         if constexpr (MODEL == MODEL_MIPS) {
             mips_gradients<VEC>(rm, rc, rn, gx, gy);
@@ -818,7 +852,7 @@ __device__ __forceinline__ void direct_strip(const StepArgs &a, const LatDesc *d
     if constexpr (SAMPLE) observe_flush<VEC>(dp->colp, dp->scal, nx, s, sy, x0, valid, obs, lane);
 }
 
-template <int MODEL, int ST, int VEC, bool SAMPLE, int NOISE>
+template <int MODEL, int ST, int VEC, bool SAMPLE, int NOISE, bool RAGGED>
 __global__ void __launch_bounds__(256, direct_min_blocks<MODEL, ST, VEC, SAMPLE>()) step_kernel(const StepArgs a)
 {
     wait_for_previous();
@@ -826,7 +860,7 @@ __global__ void __launch_bounds__(256, direct_min_blocks<MODEL, ST, VEC, SAMPLE>
     const LatDesc *dp = a.desc + find_lattice(a.desc, a.nlat, blockIdx.x);
     const int s = (blockIdx.x - dp->block_begin) * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (s >= dp->nsx * dp->nsy) return;  // whole warp leaves together
-    direct_strip<MODEL, ST, VEC, SAMPLE, NOISE>(a, dp, s, a.src, *a.t_ptr + a.k);
+    direct_strip<MODEL, ST, VEC, SAMPLE, NOISE, RAGGED>(a, dp, s, a.src, *a.t_ptr + a.k);
 }
 
 // Observable partials of the stored state without stepping (same strip

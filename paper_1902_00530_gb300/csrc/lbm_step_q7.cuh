@@ -83,6 +83,21 @@ __device__ __forceinline__ void pull_row7(const typename Store<ST>::T *base, siz
     pull_pop7<ST, VEC, 6, P>(base + 6 * plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q7(6), f[6]);
 }
 
+// See wrap_partial: the populations pulled from x + 1 of a row of parity P.
+template <int ST, int VEC, int P>
+__device__ __forceinline__ void wrap_partial7(const typename Store<ST>::T *base, size_t plane, int y, int ny, int pitch,
+                                              int nv, const Shift3 &sh, float f[7][VEC])
+{
+#pragma unroll
+    for (int i = 1; i < 7; ++i) {
+        if (q7_src_dx(i, P) != 1) continue;
+        const float v = load_one<ST>(base + i * plane + (size_t)wrap_once(y + q7_src_dy(i), ny) * pitch, sh.q7(i));
+#pragma unroll
+        for (int j = 0; j < VEC - 1; ++j)
+            if (j == nv - 1) f[i][j] = v;
+    }
+}
+
 __device__ __forceinline__ float density7(const float f[7])
 {
     return __fadd_rn(__fadd_rn(__fadd_rn(f[0], f[1]), __fadd_rn(f[2], f[3])),
@@ -96,7 +111,7 @@ __device__ __forceinline__ float density7_at(const float f[7][VEC], int j)
     return density7(v);
 }
 
-template <int ST, int VEC, int P>
+template <int ST, int VEC, int P, bool RAGGED>
 __device__ __forceinline__ void density_window7(const float f[7][VEC], const typename Store<ST>::T *base,
                                                 size_t plane, int y, int nx, int ny, int pitch, int x0, bool valid,
                                                 bool last, int lane, const Shift3 &sh, float r[VEC + 2])
@@ -124,6 +139,7 @@ __device__ __forceinline__ void density_window7(const float f[7][VEC], const typ
     if (last) right = halo_right;
     r[0] = left;
     r[VEC + 1] = right;
+    if (RAGGED && valid && x0 + VEC > nx) wrap_partial_window<VEC>(nx - x0, right, r);
 }
 
 // The Sec. 3 stencils at the lane's sites of a row of parity P, from the
@@ -251,19 +267,22 @@ struct Q7Walk {
     ObserveSums<VEC> obs;
 };
 
-template <int MODEL, int ST, int VEC, bool SAMPLE, int P>
+template <int MODEL, int ST, int VEC, bool SAMPLE, int P, bool RAGGED>
 __device__ __forceinline__ void q7_row(Q7Walk<VEC> &w, int y, const typename Store<ST>::T *src,
                                        typename Store<ST>::T *dst, size_t plane, int nx, int ny, int pitch, int x0,
                                        bool valid, bool last, int lane, const Shift3 &sh, const SiteParams &d, bool noise,
                                        uint32_t t, uint32_t id, const uint32_t *rk, double *rowp)
 {
     float fn[7][VEC];
+    const bool partial = RAGGED && valid && x0 + VEC > nx;
     if constexpr (MODEL == MODEL_MIPS) {
         const int yn = wrap_once(y + 1, ny);
         pull_row7<ST, VEC, 1 - P>(src, plane, yn, ny, nx, pitch, x0, valid, last, lane, sh, fn);
-        density_window7<ST, VEC, 1 - P>(fn, src, plane, yn, nx, ny, pitch, x0, valid, last, lane, sh, w.rn);
+        if (partial) wrap_partial7<ST, VEC, 1 - P>(src, plane, yn, ny, pitch, nx - x0, sh, fn);
+        density_window7<ST, VEC, 1 - P, RAGGED>(fn, src, plane, yn, nx, ny, pitch, x0, valid, last, lane, sh, w.rn);
     } else {
         pull_row7<ST, VEC, P>(src, plane, y, ny, nx, pitch, x0, valid, last, lane, sh, w.fc);
+        if (partial) wrap_partial7<ST, VEC, P>(src, plane, y, ny, pitch, nx - x0, sh, w.fc);
     }
     float gx[VEC], gy[VEC];
     if constexpr (MODEL == MODEL_MIPS) {
@@ -313,7 +332,7 @@ __device__ __forceinline__ void q7_row(Q7Walk<VEC> &w, int y, const typename Sto
 // One warp's strip s (< nsx nsy) of D2Q7 lattice dp for the step at time t,
 // read from buffer `src` and written to the other: the body of the direct
 // D2Q7 kernel, shared by the per-step launch and the persistent launch.
-template <int MODEL, int ST, int VEC, bool SAMPLE, int NOISE>
+template <int MODEL, int ST, int VEC, bool SAMPLE, int NOISE, bool RAGGED = false>
 __device__ __forceinline__ void direct_strip_q7(const StepArgs &a, const LatDesc *dp, int s, int src_buf, uint32_t t)
 {
     using T = typename Store<ST>::T;
@@ -338,23 +357,26 @@ __device__ __forceinline__ void direct_strip_q7(const StepArgs &a, const LatDesc
     Q7Walk<VEC> w;
     if constexpr (SAMPLE) w.obs.clear();
     if constexpr (MODEL == MODEL_MIPS) {
+        const bool partial = RAGGED && valid && x0 + VEC > nx;
         float tmp[7][VEC];
         const int yp = wrap_once(y_begin - 1, ny);  // odd
         pull_row7<ST, VEC, 1>(src, plane, yp, ny, nx, pitch, x0, valid, last, lane, sh, tmp);
-        density_window7<ST, VEC, 1>(tmp, src, plane, yp, nx, ny, pitch, x0, valid, last, lane, sh, w.rm);
+        if (partial) wrap_partial7<ST, VEC, 1>(src, plane, yp, ny, pitch, nx - x0, sh, tmp);
+        density_window7<ST, VEC, 1, RAGGED>(tmp, src, plane, yp, nx, ny, pitch, x0, valid, last, lane, sh, w.rm);
         pull_row7<ST, VEC, 0>(src, plane, y_begin, ny, nx, pitch, x0, valid, last, lane, sh, w.fc);
-        density_window7<ST, VEC, 0>(w.fc, src, plane, y_begin, nx, ny, pitch, x0, valid, last, lane, sh, w.rc);
+        if (partial) wrap_partial7<ST, VEC, 0>(src, plane, y_begin, ny, pitch, nx - x0, sh, w.fc);
+        density_window7<ST, VEC, 0, RAGGED>(w.fc, src, plane, y_begin, nx, ny, pitch, x0, valid, last, lane, sh, w.rc);
     }
     for (int y = y_begin; y < y_end; y += 2) {
-        q7_row<MODEL, ST, VEC, SAMPLE, 0>(w, y, src, dst, plane, nx, ny, pitch, x0, valid, last, lane, sh, d, noise,
+        q7_row<MODEL, ST, VEC, SAMPLE, 0, RAGGED>(w, y, src, dst, plane, nx, ny, pitch, x0, valid, last, lane, sh, d, noise,
                                           t, id, a.rk, rowp);
-        q7_row<MODEL, ST, VEC, SAMPLE, 1>(w, y + 1, src, dst, plane, nx, ny, pitch, x0, valid, last, lane, sh, d,
+        q7_row<MODEL, ST, VEC, SAMPLE, 1, RAGGED>(w, y + 1, src, dst, plane, nx, ny, pitch, x0, valid, last, lane, sh, d,
                                           noise, t, id, a.rk, rowp);
     }
     if constexpr (SAMPLE) observe_flush<VEC>(dp->colp, dp->scal, nx, s, sy, x0, valid, w.obs, lane);
 }
 
-template <int MODEL, int ST, int VEC, bool SAMPLE, int NOISE>
+template <int MODEL, int ST, int VEC, bool SAMPLE, int NOISE, bool RAGGED>
 __global__ void __launch_bounds__(256) step_kernel_q7(const StepArgs a)
 {
     wait_for_previous();
@@ -362,7 +384,7 @@ __global__ void __launch_bounds__(256) step_kernel_q7(const StepArgs a)
     const LatDesc *dp = a.desc + find_lattice(a.desc, a.nlat, blockIdx.x);
     const int s = (blockIdx.x - dp->block_begin) * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (s >= dp->nsx * dp->nsy) return;  // whole warp leaves together
-    direct_strip_q7<MODEL, ST, VEC, SAMPLE, NOISE>(a, dp, s, a.src, *a.t_ptr + a.k);
+    direct_strip_q7<MODEL, ST, VEC, SAMPLE, NOISE, RAGGED>(a, dp, s, a.src, *a.t_ptr + a.k);
 }
 
 // The D2Q7 strip update of the persistent launch (lbm_step_persistent.cuh).

@@ -513,7 +513,12 @@ template <int MODEL, int ST, int VEC, bool SAMPLE, int NOISE>
 static cudaError_t launch_one(int kind, const StepArgs &a, int blocks, int warps, cudaStream_t stream)
 {
     if (kind == 1) return launch_one_staged<MODEL, ST, VEC, SAMPLE, NOISE>(a, blocks, warps, stream);
-    return launch_dependent(step_kernel<MODEL, ST, VEC, SAMPLE, NOISE>, dim3(blocks), dim3(warps * 32), 0, stream, a);
+    const dim3 grid(blocks), block(warps * 32);
+    if constexpr (!SAMPLE && VEC > 1) {
+        if (a.ragged)
+            return launch_dependent(step_kernel<MODEL, ST, VEC, SAMPLE, NOISE, true>, grid, block, 0, stream, a);
+    }
+    return launch_dependent(step_kernel<MODEL, ST, VEC, SAMPLE, NOISE, false>, grid, block, 0, stream, a);
 }
 
 // Sample steps (one in sample_every) decide the noise at run time; the other

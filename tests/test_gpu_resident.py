@@ -111,3 +111,26 @@ def test_lattice_beyond_a_cluster_stays_per_step():
     """A lattice whose two buffers exceed the shared memory of sixteen blocks."""
     la = _run("auto", "f32", [(400, 400, "CIL_RHO1", {}, C2, "d2q9")], (6,))[1]
     assert la == [7]  # six steps and the time advance
+
+
+@pytest.mark.parametrize("storage", ["f32", "f16s"])
+@pytest.mark.parametrize("preset,vs", [("MIPS_RHO1", "d2q9"), ("CIL_RHO1", "d2q9"), ("PASSIVE", "d2q9"),
+                                       ("MIPS_Q7_RHO1", "d2q7"), ("CIL_Q7_RHO1", "d2q7")])
+@pytest.mark.parametrize("size", [(1021, 402), (1022, 300), (1923, 130), (257, 640), (4099, 514)],
+                         ids=lambda s: f"{s[0]}x{s[1]}")
+def test_tuned_plain_shapes_equal_one_site_per_thread(size, preset, vs, storage):
+    """Widths that no vector divides, beyond the resident launch: the tuned
+    shape of plain steps (short strips, vectors that a row ends inside)
+    against one site per thread in 8-row strips."""
+    from paper_1902_00530_gb300 import Lattice, Simulation
+    model, d = split_preset(preset)
+    out = []
+    for fixed in (False, True):
+        sim = Simulation([Lattice(*size, storage, 3, vs)], [model], [d])
+        if fixed:
+            sim.set_tuning(1, 1, 8, 4, 0)
+        sim.init(SEED, [C2])
+        sim.step(5)
+        out.append(sim.get_state(host=True).numpy())
+        sim.close()
+    np.testing.assert_array_equal(out[0], out[1])
