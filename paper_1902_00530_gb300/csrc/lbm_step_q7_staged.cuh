@@ -205,38 +205,37 @@ __global__ void __maxnreg__(staged_max_regs<VEC>()) step_staged_kernel_q7(const 
     constexpr bool MIPS = (MODEL == MODEL_MIPS);
     const int q_first_row = MIPS ? y_begin - 1 : y_begin;
     const int nq = (y_end - y_begin) + (MIPS ? 2 : 0);
-    auto stage_ptr = [&](int q) { return ring + (size_t)(q % S) * stage_elems; };
+    auto stage_ptr = [&](RingPos r) { return ring + (size_t)r.slot * stage_elems; };
     bool ok = true;
     auto fail = [&]() {
         ok = false;
         if (lane == 0) atomicOr(a.err, (unsigned)DEVERR_TIMEOUT);
     };
     int issued = 0;  // rows issued (warp 0)
-    auto issue = [&]() {
-        const int k = issued % S;
-        issue_row7<ST, VEC>(ring + (size_t)k * stage_elems, sg, &full[k], src, plane, pitch, nx, ny, xs, xe,
+    auto issue = [&](int slot) {
+        issue_row7<ST, VEC>(ring + (size_t)slot * stage_elems, sg, &full[slot], src, plane, pitch, nx, ny, xs, xe,
                             wrap_once(q_first_row + issued, ny), lane);
         ++issued;
     };
     if (leader)
-        while (issued < S && issued < nq) issue();
+        while (issued < S && issued < nq) issue(issued);
 
     // Row q is consumed by this warp; warp 0 refills its buffer with row q + S
     // once every warp has (a single warp needs no barrier for that).
-    auto release = [&](int q) {
+    auto release = [&](RingPos r) {
         __syncwarp();
-        if (blk.nact == 1) {
-            if (ok && issued < nq) issue();
+        if (blk.nact == 1) {  // a single warp: its own reads are all there is to wait for
+            if (ok && issued < nq) issue(r.slot);
             return;
         }
-        if (lane == 0) mbar_arrive(&empty[q % S]);
+        if (lane == 0) mbar_arrive(&empty[r.slot]);
         if (leader && ok && issued < nq) {
-            if (!stage_wait(&empty[q % S], (uint32_t)((q / S) & 1))) fail();
-            else issue();
+            if (!stage_wait(&empty[r.slot], r.phase)) fail();
+            else issue(r.slot);
         }
     };
-    auto wait_q = [&](int q) {
-        if (ok && !stage_wait(&full[q % S], (uint32_t)((q / S) & 1))) fail();
+    auto wait_row = [&](RingPos r) {
+        if (ok && !stage_wait(&full[r.slot], r.phase)) fail();
         return ok;
     };
 
@@ -245,41 +244,53 @@ __global__ void __maxnreg__(staged_max_regs<VEC>()) step_staged_kernel_q7(const 
     double *rowp = dp->rowp + (size_t)sx * ny;
 
     float rm[VEC + 2], rc[VEC + 2], rn[VEC + 2];
-    int q = 0;
+    int q = 0;            // row to update next, and its place in the ring
+    RingPos at{0, 0u};
     if constexpr (MIPS) {
-        if (wait_q(0)) {
-            stage_density_window7<ST, VEC, 1>(stage_ptr(0), sg, b, sh, lane, rm);  // row y_begin-1: odd
-            release(0);
+        if (wait_row(at)) {
+            stage_density_window7<ST, VEC, 1>(stage_ptr(at), sg, b, sh, lane, rm);  // row y_begin-1: odd
+            release(at);
         }
         q = 1;
-        if (wait_q(1)) {
-            stage_density_window7<ST, VEC, 0>(stage_ptr(1), sg, b, sh, lane, rc, CONV ? cv(1) : nullptr, G::W);
-            if constexpr (CONV) release(1);
+        at = at.next(S);
+        if (wait_row(at)) {
+            stage_density_window7<ST, VEC, 0>(stage_ptr(at), sg, b, sh, lane, rc, CONV ? cv(1) : nullptr, G::W);
+            if constexpr (CONV) release(at);
         }
     }
 
     // one row of parity P; returns false if a wait gave up
     auto do_row = [&](auto parity, int y) -> bool {
         constexpr int P = decltype(parity)::value;
-        const int qc = q;
+        const RingPos cur = at;
+        at = at.next(S);
         float f[7][VEC];
         if constexpr (CONV) {
-            if (!wait_q(qc + 1)) return false;
-            stage_density_window7<ST, VEC, 1 - P>(stage_ptr(qc + 1), sg, b, sh, lane, rn, cv(qc + 1), G::W);
-            release(qc + 1);
+            if (!wait_row(at)) {
+                at = cur;
+                return false;
+            }
+            stage_density_window7<ST, VEC, 1 - P>(stage_ptr(at), sg, b, sh, lane, rn, cv(q + 1), G::W);
+            release(at);
 #pragma unroll
-            for (int i = 0; i < 7; ++i) get_f32<VEC>(cv(qc) + i * G::W, f[i]);
+            for (int i = 0; i < 7; ++i) get_f32<VEC>(cv(q) + i * G::W, f[i]);
         } else if constexpr (MIPS) {
-            if (!wait_q(qc + 1)) return false;
-            stage_density_window7<ST, VEC, 1 - P>(stage_ptr(qc + 1), sg, b, sh, lane, rn);
-            stage_row7<ST, VEC, P>(stage_ptr(qc), sg, b, sh, f);
-            release(qc);
+            if (!wait_row(at)) {
+                at = cur;
+                return false;
+            }
+            stage_density_window7<ST, VEC, 1 - P>(stage_ptr(at), sg, b, sh, lane, rn);
+            stage_row7<ST, VEC, P>(stage_ptr(cur), sg, b, sh, f);
+            release(cur);
         } else {
-            if (!wait_q(qc)) return false;
-            stage_row7<ST, VEC, P>(stage_ptr(qc), sg, b, sh, f);
-            release(qc);
+            if (!wait_row(cur)) {
+                at = cur;
+                return false;
+            }
+            stage_row7<ST, VEC, P>(stage_ptr(cur), sg, b, sh, f);
+            release(cur);
         }
-        q = qc + 1;
+        ++q;
         float gx[VEC], gy[VEC];
         if constexpr (MIPS) {
             mips_gradients7<VEC, P>(rm, rc, rn, gx, gy);
@@ -330,8 +341,8 @@ __global__ void __maxnreg__(staged_max_regs<VEC>()) step_staged_kernel_q7(const 
     if (leader) {
         // the copies warp 0 issued must land before the block's shared memory is
         // released: wait for the rows it has not waited for itself (bounded)
-        for (int qq = q + (MIPS ? 1 : 0); qq < issued; ++qq)
-            (void)stage_wait(&full[qq % S], (uint32_t)((qq / S) & 1));
+        RingPos r = MIPS ? at.next(S) : at;
+        for (int qq = q + (MIPS ? 1 : 0); qq < issued; ++qq, r = r.next(S)) (void)stage_wait(&full[r.slot], r.phase);
     }
     if (!ok) return;
     if constexpr (SAMPLE) observe_flush<VEC>(dp->colp, dp->scal, nx, s, sy, x0, valid, obs, lane);
