@@ -189,12 +189,15 @@ lbm_status lbm_observable_series(lbm_ctx *ctx, int32_t lattice, lbm_obs *out, in
 
 /* Copy lattice `lattice`'s populations out as dense FP32 [Q][ny][nx]; dst is a
  * host pointer if dst_is_host, else a device pointer.  16-bit storage is
- * expanded to f_i = w_i rho0 + s_i.  Syncs. */
+ * expanded to f_i = w_i rho0 + s_i (for a host dst on the device, through the
+ * lattice's spare population buffer; a pinned dst is copied to at the host
+ * link's speed).  Syncs. */
 lbm_status lbm_get_state(lbm_ctx *ctx, int32_t lattice, float *dst, int32_t dst_is_host);
 
 /* Replace lattice `lattice`'s populations by dense FP32 [Q][ny][nx] from src
  * (host if src_is_host, else device).  16-bit storage stores s_i = f_i -
- * w_i rho0 rounded to nearest.  Does not change t.  Syncs. */
+ * w_i rho0 rounded to nearest (from the host too, the device converting).
+ * Does not change t.  Syncs. */
 lbm_status lbm_set_state(lbm_ctx *ctx, int32_t lattice, const float *src, int32_t src_is_host);
 
 /* Change the mean density of lattice `lattice` (-1: every lattice) without
@@ -242,7 +245,11 @@ lbm_status lbm_set_tuning(lbm_ctx *ctx, int32_t mode, int32_t vec, int32_t rows,
 lbm_status lbm_tune(lbm_ctx *ctx);
 
 /* The launch shape in use for lattice `lattice`: vec, rows, warps per block,
- * stages (0 = direct-load kernel). */
+ * stages (0 = direct-load kernel).  Under automatic tuning this is the shape of
+ * steps that take a sample; steps that do not may run a direct shape that
+ * lbm_set_tuning does not offer (strips of 1, 2 or 4 rows, vectors that do not
+ * divide nx), or one of the launch forms of lbm_set_persistent, where the tuner
+ * found those faster.  States are the same in every shape and form. */
 lbm_status lbm_get_tuning(const lbm_ctx *ctx, int32_t lattice, int32_t *vec, int32_t *rows,
                           int32_t *warps, int32_t *stages);
 
@@ -283,7 +290,7 @@ lbm_status lbm_set_graphs(lbm_ctx *ctx, int32_t enabled);
  * launch: one cluster per lattice keeps it on chip for a whole stretch of
  * steps, reading and writing device memory once per stretch.  It is kept where
  * it is faster than the forms above (measured: the paper's 90 x 30 MIPS box at
- * 1.2 us per step against 12.4, 32 boxes of 180 x 60 at 6 us against 12);
+ * 1.3 us per step against 12.4, 32 boxes of 180 x 60 at 4.4 us against 12);
  * lbm_get_persistent reports 0 for such a group, and its sample steps and
  * single steps launch once per step.  Modes 0 and 1 and fixed shapes never use it.
  * The waits are bounded (about 1 s, then the error flag is raised and the call

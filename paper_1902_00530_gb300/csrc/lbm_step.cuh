@@ -141,7 +141,7 @@ __device__ __forceinline__ void wrap_partial(const typename Store<ST>::T *base, 
         const float v = load_one<ST>(base + i * plane + (size_t)wrap_once(y - vy(i), ny) * pitch, sh.q9(i));
 #pragma unroll
         for (int j = 0; j < VEC - 1; ++j)
-            if (j == nv - 1) f[i][j] = v;
+            f[i][j] = j == nv - 1 ? v : f[i][j];
     }
 }
 // The same for a row's density window (r[k] is site x0 + k - 1).
@@ -149,7 +149,7 @@ template <int VEC> __device__ __forceinline__ void wrap_partial_window(int nv, f
 {
 #pragma unroll
     for (int k = 2; k < VEC + 1; ++k)
-        if (k == nv + 1) r[k] = right;
+        r[k] = k == nv + 1 ? right : r[k];
 }
 
 template <int VEC>
@@ -738,8 +738,12 @@ template <int MODEL, int ST, int VEC, bool SAMPLE> constexpr int direct_min_bloc
 // shared by the per-step launch and the persistent launch.  RAGGED: VEC need not
 // divide nx (see wrap_partial; a form of its own, since the test for it in every
 // row cost the others 5 to 9 %: 1024^2 CIL 14.3 -> 15.1 us, MIPS 21.9 -> 24.6).
-template <int MODEL, int ST, int VEC, bool SAMPLE, int NOISE, bool RAGGED = false>
-__device__ __forceinline__ void direct_strip(const StepArgs &a, const LatDesc *dp, int s, int src_buf, uint32_t t)
+// time() gives the step's time, and is called before the first access to
+// anything another launch writes: the per-step launch waits there for the one
+// before it, having read its lattice's descriptor meanwhile (the buffers'
+// addresses are read after it, so no load of theirs can be moved ahead of it).
+template <int MODEL, int ST, int VEC, bool SAMPLE, int NOISE, bool RAGGED = false, typename Time>
+__device__ __forceinline__ void direct_strip(const StepArgs &a, const LatDesc *dp, int s, int src_buf, Time time)
 {
     using T = typename Store<ST>::T;
     const int lane = threadIdx.x & 31;
@@ -756,10 +760,11 @@ __device__ __forceinline__ void direct_strip(const StepArgs &a, const LatDesc *d
     const uint32_t plane32 = (uint32_t)plane;  // q ny pitch <= 2^32 (host check) where used
     // 64-bit pointer steps only in the copy-bound noise-free kernels (see pull_pop_wide)
     constexpr bool WIDE = MODEL != MODEL_MIPS && NOISE == 0 && !SAMPLE;
-    const T *src = reinterpret_cast<const T *>(dp->f[src_buf]);
-    T *dst = reinterpret_cast<T *>(dp->f[src_buf ^ 1]);
     const Shift3 sh = load_shift(dp);
     const uint32_t id = (uint32_t)dp->id;
+    const uint32_t t = time();
+    const T *src = reinterpret_cast<const T *>(dp->f[src_buf]);
+    T *dst = reinterpret_cast<T *>(dp->f[src_buf ^ 1]);
     const bool noise = NOISE == 2 ? d.sigma_q > 0.f : NOISE == 1;
 
     ObserveSums<VEC> obs;
@@ -855,12 +860,14 @@ __device__ __forceinline__ void direct_strip(const StepArgs &a, const LatDesc *d
 template <int MODEL, int ST, int VEC, bool SAMPLE, int NOISE, bool RAGGED>
 __global__ void __launch_bounds__(256, direct_min_blocks<MODEL, ST, VEC, SAMPLE>()) step_kernel(const StepArgs a)
 {
-    wait_for_previous();
-    allow_dependents();
     const LatDesc *dp = a.desc + find_lattice(a.desc, a.nlat, blockIdx.x);
     const int s = (blockIdx.x - dp->block_begin) * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (s >= dp->nsx * dp->nsy) return;  // whole warp leaves together
-    direct_strip<MODEL, ST, VEC, SAMPLE, NOISE, RAGGED>(a, dp, s, a.src, *a.t_ptr + a.k);
+    direct_strip<MODEL, ST, VEC, SAMPLE, NOISE, RAGGED>(a, dp, s, a.src, [&] {
+        wait_for_previous();
+        return *a.t_ptr + a.k;
+    });
+    allow_dependents();
 }
 
 // Observable partials of the stored state without stepping (same strip

@@ -94,7 +94,7 @@ __device__ __forceinline__ void wrap_partial7(const typename Store<ST>::T *base,
         const float v = load_one<ST>(base + i * plane + (size_t)wrap_once(y + q7_src_dy(i), ny) * pitch, sh.q7(i));
 #pragma unroll
         for (int j = 0; j < VEC - 1; ++j)
-            if (j == nv - 1) f[i][j] = v;
+            f[i][j] = j == nv - 1 ? v : f[i][j];
     }
 }
 
@@ -332,8 +332,9 @@ __device__ __forceinline__ void q7_row(Q7Walk<VEC> &w, int y, const typename Sto
 // One warp's strip s (< nsx nsy) of D2Q7 lattice dp for the step at time t,
 // read from buffer `src` and written to the other: the body of the direct
 // D2Q7 kernel, shared by the per-step launch and the persistent launch.
-template <int MODEL, int ST, int VEC, bool SAMPLE, int NOISE, bool RAGGED = false>
-__device__ __forceinline__ void direct_strip_q7(const StepArgs &a, const LatDesc *dp, int s, int src_buf, uint32_t t)
+// time() as in direct_strip.
+template <int MODEL, int ST, int VEC, bool SAMPLE, int NOISE, bool RAGGED = false, typename Time>
+__device__ __forceinline__ void direct_strip_q7(const StepArgs &a, const LatDesc *dp, int s, int src_buf, Time time)
 {
     using T = typename Store<ST>::T;
     const int lane = threadIdx.x & 31;
@@ -347,10 +348,11 @@ __device__ __forceinline__ void direct_strip_q7(const StepArgs &a, const LatDesc
     // rows and ny are even, so every strip starts on an even row and holds whole (even, odd) pairs
     const int y_begin = sy * rows, y_end = min(y_begin + rows, ny);
     const size_t plane = (size_t)ny * pitch;
-    const T *src = reinterpret_cast<const T *>(dp->f[src_buf]);
-    T *dst = reinterpret_cast<T *>(dp->f[src_buf ^ 1]);
     const Shift3 sh = load_shift(dp);
     const uint32_t id = (uint32_t)dp->id;
+    const uint32_t t = time();
+    const T *src = reinterpret_cast<const T *>(dp->f[src_buf]);
+    T *dst = reinterpret_cast<T *>(dp->f[src_buf ^ 1]);
     const bool noise = NOISE == 2 ? d.sigma_q > 0.f : NOISE == 1;  // as in step_kernel
     double *rowp = dp->rowp + (size_t)sx * ny;
 
@@ -379,12 +381,14 @@ __device__ __forceinline__ void direct_strip_q7(const StepArgs &a, const LatDesc
 template <int MODEL, int ST, int VEC, bool SAMPLE, int NOISE, bool RAGGED>
 __global__ void __launch_bounds__(256) step_kernel_q7(const StepArgs a)
 {
-    wait_for_previous();
-    allow_dependents();
     const LatDesc *dp = a.desc + find_lattice(a.desc, a.nlat, blockIdx.x);
     const int s = (blockIdx.x - dp->block_begin) * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (s >= dp->nsx * dp->nsy) return;  // whole warp leaves together
-    direct_strip_q7<MODEL, ST, VEC, SAMPLE, NOISE, RAGGED>(a, dp, s, a.src, *a.t_ptr + a.k);
+    direct_strip_q7<MODEL, ST, VEC, SAMPLE, NOISE, RAGGED>(a, dp, s, a.src, [&] {
+        wait_for_previous();
+        return *a.t_ptr + a.k;
+    });
+    allow_dependents();
 }
 
 // The D2Q7 strip update of the persistent launch (lbm_step_persistent.cuh).
@@ -392,7 +396,7 @@ template <> struct PersistStrip<7> {
     template <int MODEL, int ST, int VEC, int NOISE>
     static __device__ __forceinline__ void run(const StepArgs &a, const LatDesc *dp, int s, int src, uint32_t t)
     {
-        direct_strip_q7<MODEL, ST, VEC, false, NOISE>(a, dp, s, src, t);
+        direct_strip_q7<MODEL, ST, VEC, false, NOISE>(a, dp, s, src, [t] { return t; });
     }
 };
 
