@@ -39,7 +39,7 @@ constexpr int TUNE_STEPS_MAX = 256;
 // the tuner's second look: at most so many candidates within this factor of the fastest, so often
 constexpr size_t TUNE_FINALISTS = 5;
 constexpr float TUNE_FINAL_MARGIN = 1.08f;
-constexpr int TUNE_FINAL_REPS = 3;
+constexpr int TUNE_FINAL_REPS = 2;
 // Mode 2 considers persistent launches only for groups with at least this
 // many sites per step.  Below it a step's items cannot fill the GPU in either
 // form and the persistent launch's dependency waits cost more than a launch
@@ -1013,7 +1013,7 @@ lbm_status tune_group(lbm_ctx *c, GroupHost &g, std::vector<Choice> *alts)
             return LBM_OK;
         }
         float ms = 0.f;
-        st = time_form(steps, &ms);
+        st = time_form(steps, &ms, 0.5f * TUNE_MIN_MS);  // the final look decides between the nearly equal
         if (st != LBM_OK) return st;
         timed.push_back({ms, now});
         if (ms < best) {
@@ -1023,6 +1023,18 @@ lbm_status tune_group(lbm_ctx *c, GroupHost &g, std::vector<Choice> *alts)
         return LBM_OK;
     };
     lbm_status st = LBM_OK;
+    // mode 2: the resident launch where the lattices fit on chip
+    if (c->persist_mode == 2 && best_step < 1e29f && plan_resident(c, g)) {
+        const Choice before = b;
+        Choice now = b.persist ? bstep : b;
+        now.resident = true;
+        st = consider(now, TUNE_STEPS_PERSIST);
+        if (st != LBM_OK) return st;
+        if (b.resident) alts->push_back(before);
+    }
+    // A resident launch several times faster than any other form leaves only single
+    // steps to the shapes below: not worth their timings.
+    const bool settled = b.resident && best * 3.f < best_step;
     // Direct shapes for the steps without a sample that the shape of sample steps
     // cannot have.  Strips of fewer than 8 rows (which would size the scratch of
     // the partials): a warp walks its rows one after the other, so in a lattice
@@ -1031,7 +1043,7 @@ lbm_status tune_group(lbm_ctx *c, GroupHost &g, std::vector<Choice> *alts)
     // strips, 4.5 in shorter ones.  Vectors that do not divide nx (a row then
     // ends inside a lane's vector, wrap_partial): one site per thread costs an odd
     // width up to twice the instructions per site.
-    if (c->persist_mode != 1 && best_step < 1e29f && direct) {
+    if (c->persist_mode != 1 && best_step < 1e29f && direct && !settled) {
         for (int v : all_v) {
             if (!allowed_vec(g.storage, v)) continue;
             bool divides = true;
@@ -1049,15 +1061,6 @@ lbm_status tune_group(lbm_ctx *c, GroupHost &g, std::vector<Choice> *alts)
         }
     }
     if (b.plain.rows > 0) alts->push_back(bstep);
-    // mode 2: the resident launch where the lattices fit on chip
-    if (c->persist_mode == 2 && best_step < 1e29f && plan_resident(c, g)) {
-        const Choice before = b;
-        Choice now = b.persist ? bstep : b;
-        now.resident = true;
-        st = consider(now, TUNE_STEPS_PERSIST);
-        if (st != LBM_OK) return st;
-        if (b.resident) alts->push_back(before);
-    }
     // The short timings differ by several percent from run to run: the few
     // fastest are timed again, in turn, and the fastest of those is kept.
     std::sort(timed.begin(), timed.end(), [](const auto &x, const auto &y) { return x.first < y.first; });
@@ -1071,7 +1074,7 @@ lbm_status tune_group(lbm_ctx *c, GroupHost &g, std::vector<Choice> *alts)
             if (st != LBM_OK) return st;
             float ms = 0.f;
             st = time_form(resident_ok(c, g) || persistent_ok(c, g) ? TUNE_STEPS_PERSIST : TUNE_STEPS, &ms,
-                           4 * TUNE_MIN_MS);
+                           2 * TUNE_MIN_MS);
             if (st != LBM_OK) return st;
             again[k] = std::min(again[k], ms);
         }
