@@ -3,7 +3,8 @@
 // The context holds host descriptors only; all device memory (population
 // buffers and scratch) belongs to the caller.  Scratch layout (256-byte
 // aligned regions): control words (step counter t, error flag), per-lattice
-// counters, descriptor tables (all lattices, then one table per launch group),
+// counters, descriptor tables (all lattices, then two per launch group: its shape's
+// and its plain steps'),
 // per launch group the persistent launch's work counter, strip-row progress
 // counters and lattice-group table, initial-state specs, and per lattice the
 // reduction partials, the finaliser partials, the observable ring and the
@@ -853,8 +854,10 @@ void choose(GroupHost &g, const Choice &ch)
 // lattice) with the least estimated time per step, if any fits.  A step takes
 // a latency (barrier, one pass of dependent arithmetic) plus the sites an SM
 // has to update, in waves of the clusters that fit the GPU at once.  In SM
-// cycles, RES_STEP_CYCLES and RES_SITE_CYCLES are the measured latency of a
-// step of a nearly empty band and the time per site of a full one.
+// cycles, RES_STEP_CYCLES and RES_SITE_CYCLES stand for the latency of a step
+// of a nearly empty band and the time per site of a full one (measured 2700 for
+// 90 x 30 MIPS with its extra barrier and density pass, and 3.4 for 32 boxes of
+// 180 x 60; only their order decides, waves first, then the cluster size).
 constexpr double RES_STEP_CYCLES = 1000.0, RES_SITE_CYCLES = 4.0;
 
 bool plan_resident(const lbm_ctx *c, GroupHost &g)

@@ -92,7 +92,8 @@ __global__ void init_kernel(const LatDesc *desc, const InitSpecDev *specs, int d
 // one element per thread and 64-bit divisions for its plane, row and column,
 // 4096^2 BF16 took 620 us out, 736 us in, 603 us for a density step and 161 us
 // for the moments; the bytes take 134, 134, 89 and 74 us.  FP32 went through
-// cudaMemcpy2D: 608 us against 178.)
+// cudaMemcpy2D: 608 us against 178.  Whole calls of these kernels now: BF16 181 us
+// out, 155 in, 115 for a density step, 106 for the moments; FP32 186 out, 201 in.)
 // ---------------------------------------------------------------------------
 constexpr int EXCHANGE_ROWS = 4;
 
@@ -266,8 +267,8 @@ __global__ void __launch_bounds__(256) add_density_kernel(const LatDesc *desc, i
 // strips: 128 loads a lane, not 1024 in a row), the sums of each kind are
 // reduced by their own warps at the same time (an FP64 addition takes a
 // warp's scheduler 64 cycles), and the record's divisions and square roots are
-// formed by eight lanes at once.  (ncu, 4096^2: 44 -> 16 us; 32 lattices of
-// 180 x 60: 20.5 -> 12.1 us.)
+// formed by eight lanes at once.  (ncu, cold caches: 4096^2 44 -> 19 us; 32 lattices
+// of 180 x 60 20.5 -> 15.6 us.)
 //
 // An on-demand call (to_ring 0) wants one lattice's record on the host, and
 // the error word after every lattice's sums: the last lattice to finish writes
