@@ -188,10 +188,11 @@ lbm_status lbm_observable_series(lbm_ctx *ctx, int32_t lattice, lbm_obs *out, in
                                  int32_t *n_out);
 
 /* Copy lattice `lattice`'s populations out as dense FP32 [Q][ny][nx]; dst is a
- * host pointer if dst_is_host, else a device pointer.  16-bit storage is
- * expanded to f_i = w_i rho0 + s_i (for a host dst on the device, through the
- * lattice's spare population buffer; a pinned dst is copied to at the host
- * link's speed).  Syncs. */
+ * host pointer if dst_is_host, else a device pointer (of this GPU, or of another
+ * one the copy engine reaches, at any alignment).  16-bit storage is expanded to
+ * f_i = w_i rho0 + s_i (for a dst that is not this GPU's memory on the device all
+ * the same, through the lattice's spare population buffer; a pinned dst is copied
+ * to at the host link's speed).  Syncs. */
 lbm_status lbm_get_state(lbm_ctx *ctx, int32_t lattice, float *dst, int32_t dst_is_host);
 
 /* Replace lattice `lattice`'s populations by dense FP32 [Q][ny][nx] from src

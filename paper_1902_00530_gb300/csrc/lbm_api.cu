@@ -801,6 +801,23 @@ int staging_planes(const LatHost &L)
     return (int)std::min<size_t>(L.q, L.buf_bytes / ((size_t)L.lat.nx * L.lat.ny * sizeof(float)));
 }
 
+// Whether the exchange kernels may take a caller's device pointer: memory of this
+// device, or managed memory, at the alignment of a float.  Anything else (another
+// GPU's memory, which may have no peer mapping here, or a byte offset) only
+// the copy engine can reach without a fault: cudaMemcpy2D for FP32, and for 16-bit
+// storage a linear copy to or from the spare buffer, as for host memory.
+bool kernel_reaches(const void *p)
+{
+    cudaPointerAttributes at;
+    int dev = 0;
+    if (reinterpret_cast<uintptr_t>(p) % sizeof(float)) return false;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return at.type == cudaMemoryTypeManaged || (at.type == cudaMemoryTypeDevice && at.device == dev);
+}
+
 lbm_status require_ready(lbm_ctx *c, bool need_init)
 {
     if (!c) return LBM_ERR_INVALID_ARG;
@@ -1459,12 +1476,13 @@ lbm_status lbm_get_state(lbm_ctx *c, int32_t lattice, float *dst, int32_t dst_is
         return fail(c, LBM_ERR_INVALID_ARG, "bad lattice index or null output");
     const LatHost &L = c->lats[lattice];
     const int nx = L.lat.nx, ny = L.lat.ny;
-    if (!dst_is_host) {
+    if (!dst_is_host && kernel_reaches(dst)) {
         CK(launch_export(L.lat.storage, all_desc(c), lattice, 0, L.q, nx, ny, c->parity, dst, c->stream),
            "launch export");
     } else if (L.lat.storage == LBM_F32) {
         const char *src = c->state + L.state_off + (c->parity ? L.buf_bytes : 0);
-        CK(cudaMemcpy2DAsync(dst, nx * 4, src, L.pitch * 4, nx * 4, (size_t)L.q * ny, cudaMemcpyDeviceToHost, c->stream),
+        CK(cudaMemcpy2DAsync(dst, nx * 4, src, L.pitch * 4, nx * 4, (size_t)L.q * ny,
+                             dst_is_host ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice, c->stream),
            "copy populations");
     } else {
         // expanded on the device, as many populations at a time as the spare buffer holds
@@ -1475,7 +1493,9 @@ lbm_status lbm_get_state(lbm_ctx *c, int32_t lattice, float *dst, int32_t dst_is
             const int np = std::min(most, L.q - i);
             CK(launch_export(L.lat.storage, all_desc(c), lattice, i, np, nx, ny, c->parity, stage, c->stream),
                "launch export");
-            CK(cudaMemcpyAsync(dst + i * plane, stage, np * plane * sizeof(float), cudaMemcpyDeviceToHost, c->stream),
+            CK(cudaMemcpyAsync(reinterpret_cast<char *>(dst) + i * plane * sizeof(float), stage,
+                               np * plane * sizeof(float), dst_is_host ? cudaMemcpyDeviceToHost : cudaMemcpyDefault,
+                               c->stream),
                "copy populations");
         }
     }
@@ -1497,12 +1517,13 @@ lbm_status lbm_set_state(lbm_ctx *c, int32_t lattice, const float *src, int32_t 
     }
     const LatHost &L = c->lats[lattice];
     const int nx = L.lat.nx, ny = L.lat.ny;
-    if (!src_is_host) {
+    if (!src_is_host && kernel_reaches(src)) {
         CK(launch_import(L.lat.storage, all_desc(c), lattice, 0, L.q, nx, ny, c->parity, src, c->stream),
            "launch import");
     } else if (L.lat.storage == LBM_F32) {
         char *dstp = c->state + L.state_off + (c->parity ? L.buf_bytes : 0);
-        CK(cudaMemcpy2DAsync(dstp, L.pitch * 4, src, nx * 4, nx * 4, (size_t)L.q * ny, cudaMemcpyHostToDevice, c->stream),
+        CK(cudaMemcpy2DAsync(dstp, L.pitch * 4, src, nx * 4, nx * 4, (size_t)L.q * ny,
+                             src_is_host ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, c->stream),
            "copy populations");
     } else {
         const int most = staging_planes(L);
@@ -1510,7 +1531,9 @@ lbm_status lbm_set_state(lbm_ctx *c, int32_t lattice, const float *src, int32_t 
         const size_t plane = (size_t)nx * ny;
         for (int i = 0; i < L.q; i += most) {
             const int np = std::min(most, L.q - i);
-            CK(cudaMemcpyAsync(stage, src + i * plane, np * plane * sizeof(float), cudaMemcpyHostToDevice, c->stream),
+            CK(cudaMemcpyAsync(stage, reinterpret_cast<const char *>(src) + i * plane * sizeof(float),
+                               np * plane * sizeof(float), src_is_host ? cudaMemcpyHostToDevice : cudaMemcpyDefault,
+                               c->stream),
                "copy populations");
             CK(launch_import(L.lat.storage, all_desc(c), lattice, i, np, nx, ny, c->parity, stage, c->stream),
                "launch import");
