@@ -435,6 +435,15 @@ __device__ __forceinline__ float load_one(const typename Store<ST>::T *p, float 
 __device__ __forceinline__ void allow_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// Let a kernel be launched with any dynamic shared memory a block can have.  The
+// limit belongs to the kernel and not to a launch or a context, so it is always
+// set to the same value: set to a launch's own need, it could be lowered by
+// another host thread between this thread's call and its launch.
+template <typename Kernel> inline cudaError_t allow_all_smem(Kernel kern)
+{
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)STAGED_SMEM_MAX);
+}
+
 template <typename Kernel, typename... Args>
 inline cudaError_t launch_dependent(Kernel kern, dim3 grid, dim3 block, size_t smem, cudaStream_t stream, Args... args)
 {

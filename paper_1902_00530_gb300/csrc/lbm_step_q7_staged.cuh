@@ -354,7 +354,7 @@ static cudaError_t launch_one_staged7(const StepArgs &a, int blocks, int warps, 
     const size_t bytes =
         staged_smem_bytes(7, (int)sizeof(typename Store<ST>::T), VEC, warps, a.stages, staged_conv_rows(MODEL, ST));
     auto kern = step_staged_kernel_q7<MODEL, ST, VEC, SAMPLE, NOISE>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    cudaError_t e = allow_all_smem(kern);
     if (e != cudaSuccess) return e;
     kern<<<blocks, warps * 32, bytes, stream>>>(a);
     return cudaGetLastError();

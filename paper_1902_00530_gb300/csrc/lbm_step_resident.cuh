@@ -264,7 +264,7 @@ template <int Q, int MODEL, int ST>
 static cudaError_t launch_resident_one(const StepArgs &a, const ResidentArgs &p, int *clusters, cudaStream_t stream)
 {
     auto kern = step_resident_kernel<Q, MODEL, ST>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
+    cudaError_t e = allow_all_smem(kern);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
