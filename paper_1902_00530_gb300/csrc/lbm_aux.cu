@@ -373,7 +373,7 @@ __global__ void __launch_bounds__(FIN_THREADS) finalize_kernel(const LatDesc *de
     const double dev = sqrt(fmax(var, 0.0));
     const double zeta = (double)dp->B - quo;  // lane 2
     const bool finite = lane == 0 ? isfinite(mass) : lane == 1 ? isfinite(quo) : lane == 2 ? isfinite(zeta)
-                        : (lane == 3 || lane == 4) ? isfinite(var) : true;
+                        : (lane >= 3 && lane <= 5) ? isfinite(var) : true;
     const bool all_finite = __all_sync(FULL, finite);
     double rec = 0.0;
     if (lane == 0) rec = __longlong_as_double((long long)(uint32_t)(*t_ptr + k + (to_ring ? 1u : 0u)));

@@ -565,15 +565,16 @@ __device__ __forceinline__ void mips_gradients(const float rm[VEC + 2], const fl
 // ---------------------------------------------------------------------------
 // Observable sums.  The sums that cancel (rho and rho^2 in the variance, j in
 // the polar order of a nearly disordered state) must not depend on how the
-// launch shape groups sites into lanes, so they are exact to FP64 rounding from
-// a lane's first site on.  FP64 itself is far too slow for that here: a GB300
+// launch shape groups sites into lanes, so they carry more than FP32 from a
+// lane's first site on.  FP64 itself is far too slow for that here: a GB300
 // SM issues about 2 FP64 lane operations per cycle, and five FP64 additions, four
 // conversions and the FP64 row reduction per site made a 4096^2 reduction 380 us
 // (0.14 sites per cycle and SM) where its bytes take 45 to 90 us.  A lane's
-// sums are therefore unevaluated FP32 pairs h + l (48 bits: 24 bits of a
-// value leave room for 2^24 values of one magnitude; a lane adds at most a
-// few thousand, so its sums are the exact ones), added with Knuth's TwoSum and
-// turned into FP64 once per strip; what joins strips is FP64 as before.
+// sums are therefore unevaluated FP32 pairs h + l, added with Knuth's TwoSum and
+// turned into FP64 once per strip; what joins strips is FP64.  A pair has 48
+// bits against FP64's 53: sums of values of one magnitude are exact up to 2^24 of
+// them (a lane adds at most 2^15, a warp 2^20), others are rounded at 2^-48 of the sum,
+// far below the FP32 rounding of each site's rho and j.
 // ---------------------------------------------------------------------------
 struct Pair {
     float h, l;
@@ -607,15 +608,23 @@ __device__ __forceinline__ Pair pair_warp_sum(Pair a)
     return a;
 }
 
-// A lane's sums over its strip.  rho^2 = p + fma(r, r, -p) has 48 bits itself,
-// and the variance is the small difference of two such sums, so its sum is three
-// words (h + l + m).  That holds where p and its error stay in FP32's range
-// (2^-50 < rho < 2^60); rows with a density outside (an empty site, an absurd
-// scale) go to the FP64 sum r2d.
+// The pairs hold FP32's range, and a strip's sum has up to 2^20 terms (4096 rows
+// of 8 sites in 32 lanes): densities from PAIR_MAX on are summed in FP64, in the strip's
+// own column partials, which only its lane writes.  (Sums of j need no such
+// form: from |j| = 2^64 on |j|^2 is infinite, which the finaliser reports.)
+// rho^2 = p + fma(r, r, -p) has 48 bits itself, and the variance is the small
+// difference of two such sums, so its sum is three words (h + l + m).  That holds
+// where p and its error, and the 2^15 terms of a lane, stay in FP32's range
+// (SQUARE_MIN < rho < SQUARE_MAX); rows with a density outside (an empty site, an
+// absurd scale) go to the FP64 sum r2d.
+constexpr float PAIR_MAX = 0x1p96f, SQUARE_MIN = 0x1p-50f, SQUARE_MAX = 0x1p50f;
+
+// A lane's sums over its strip.
 template <int VEC> struct ObserveSums {
     Pair col[VEC], jx, jy, r2, aj;
     float r2m;
     double r2d;
+    bool wide;  // the lane has column sums in FP64 too
     __device__ __forceinline__ void clear()
     {
 #pragma unroll
@@ -623,33 +632,39 @@ template <int VEC> struct ObserveSums {
         jx = jy = r2 = aj = Pair{0.f, 0.f};
         r2m = 0.f;
         r2d = 0.0;
+        wide = false;
     }
 };
+__device__ __forceinline__ double warp_sum_f64(double v)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
+    return v;
+}
 
 // Add one stored row (sites x0..x0+VEC-1) from its moments rho and j = rho u,
-// and write the row's density total over the warp.  |j|, a sum of magnitudes,
-// is summed in FP32 over the lane's sites of the row.  Lattice-independent.
+// and write the row's density total over the warp.  cols: the lane's column partials
+// (see PAIR_MAX).  |j|, a sum of magnitudes, is summed in FP32 over the lane's sites
+// of the row.  Lattice-independent.
 template <int VEC>
 __device__ __forceinline__ void observe_moments(const float rv[VEC], const float jxv[VEC], const float jyv[VEC],
-                                                bool valid, ObserveSums<VEC> &o, double *row_out, int lane)
+                                                bool valid, ObserveSums<VEC> &o, double *cols, double *row_out, int lane)
 {
     Pair rs{0.f, 0.f};
+    bool wide = false;
     if (valid) {
         float js = 0.f;
-        bool in_range = true;
+        bool squares = true;
 #pragma unroll
         for (int j = 0; j < VEC; ++j) {
             const float r = rv[j], jx = jxv[j], jy = jyv[j];
-            pair_add(o.col[j], r);
             pair_add(o.jx, jx);
             pair_add(o.jy, jy);
-            in_range = in_range && r > 0x1p-50f && r < 0x1p60f;
+            squares = squares && r > SQUARE_MIN && r < SQUARE_MAX;
             js += sqrtf(jx * jx + jy * jy);
-            if (j == 0) rs.h = r;
-            else pair_add(rs, r);
         }
         pair_add(o.aj, js);
-        if (in_range) {
+        if (squares) {
 #pragma unroll
             for (int j = 0; j < VEC; ++j) {
                 const float p = __fmul_rn(rv[j], rv[j]);
@@ -658,17 +673,38 @@ __device__ __forceinline__ void observe_moments(const float rv[VEC], const float
             }
         } else {
 #pragma unroll
-            for (int j = 0; j < VEC; ++j) o.r2d = __fma_rn((double)rv[j], (double)rv[j], o.r2d);
+            for (int j = 0; j < VEC; ++j) {
+                o.r2d = __fma_rn((double)rv[j], (double)rv[j], o.r2d);
+                wide = wide || !(fabsf(rv[j]) < PAIR_MAX);
+            }
+        }
+        if (!wide) {
+#pragma unroll
+            for (int j = 0; j < VEC; ++j) {
+                pair_add(o.col[j], rv[j]);
+                if (j == 0) rs.h = rv[j];
+                else pair_add(rs, rv[j]);
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < VEC; ++j) cols[j] = (o.wide ? cols[j] : 0.0) + (double)rv[j];
+            o.wide = true;
         }
     }
-    rs = pair_warp_sum(rs);
-    if (lane == 0) *row_out = pair_value(rs);
+    double row = pair_value(pair_warp_sum(rs));
+    if (__any_sync(FULL, wide)) {
+        double w = 0.0;
+#pragma unroll
+        for (int j = 0; j < VEC; ++j) w += wide ? (double)rv[j] : 0.0;
+        row += warp_sum_f64(w);
+    }
+    if (lane == 0) *row_out = row;
 }
 
 // The same for a stored D2Q9 row.
 template <int VEC>
-__device__ __forceinline__ void observe_row(const float g[9][VEC], bool valid, ObserveSums<VEC> &o, double *row_out,
-                                            int lane)
+__device__ __forceinline__ void observe_row(const float g[9][VEC], bool valid, ObserveSums<VEC> &o, double *cols,
+                                            double *row_out, int lane)
 {
     float rv[VEC], jxv[VEC], jyv[VEC];
 #pragma unroll
@@ -677,7 +713,7 @@ __device__ __forceinline__ void observe_row(const float g[9][VEC], bool valid, O
         jxv[j] = (g[1][j] + g[5][j] + g[8][j]) - (g[3][j] + g[6][j] + g[7][j]);
         jyv[j] = (g[2][j] + g[5][j] + g[6][j]) - (g[4][j] + g[7][j] + g[8][j]);
     }
-    observe_moments<VEC>(rv, jxv, jyv, valid, o, row_out, lane);
+    observe_moments<VEC>(rv, jxv, jyv, valid, o, cols, row_out, lane);
 }
 
 // Write the strip's column sums and its five scalar sums (rho, j_x, j_y, rho^2,
@@ -687,19 +723,24 @@ __device__ __forceinline__ void observe_flush(double *colp, double *scal, int nx
                                               bool valid, const ObserveSums<VEC> &o, int lane)
 {
     Pair rho{0.f, 0.f};
+    double far = 0.0;  // what lies outside the pairs
 #pragma unroll
     for (int j = 0; j < VEC; ++j) pair_add(rho, o.col[j]);
     if (valid) {
+        double *const cols = colp + (size_t)sy * nx + x0;
 #pragma unroll
-        for (int j = 0; j < VEC; ++j) colp[(size_t)sy * nx + x0 + j] = pair_value(o.col[j]);
+        for (int j = 0; j < VEC; ++j) {
+            const double w = o.wide ? cols[j] : 0.0;
+            far += w;
+            cols[j] = pair_value(o.col[j]) + w;
+        }
     }
     const Pair v[4] = {pair_warp_sum(rho), pair_warp_sum(o.jx), pair_warp_sum(o.jy), pair_warp_sum(o.aj)};
-    double r2 = (pair_value(o.r2) + (double)o.r2m) + o.r2d;
-#pragma unroll
-    for (int q = 16; q > 0; q >>= 1) r2 += __shfl_xor_sync(FULL, r2, q);
+    const double r2 = warp_sum_f64((pair_value(o.r2) + (double)o.r2m) + o.r2d);
+    if (__any_sync(FULL, o.wide)) far = warp_sum_f64(far);
     if (lane == 0) {
         double *out = scal + (size_t)s * 5;
-        out[0] = pair_value(v[0]);
+        out[0] = pair_value(v[0]) + far;
         out[1] = pair_value(v[1]);
         out[2] = pair_value(v[2]);
         out[3] = r2;
@@ -844,7 +885,7 @@ __device__ __forceinline__ void direct_strip(const StepArgs &a, const LatDesc *d
 #pragma unroll
                 for (int j = 0; j < VEC; ++j)
                     g[i][j] = Store<ST>::get(Store<ST>::put(out[i][j], sh.q9(i)), sh.q9(i));
-            observe_row<VEC>(g, valid, obs, dp->rowp + (size_t)sx * ny + y, lane);
+            observe_row<VEC>(g, valid, obs, dp->colp + (size_t)sy * nx + x0, dp->rowp + (size_t)sx * ny + y, lane);
         }
         if constexpr (MODEL == MODEL_MIPS) {
 #pragma unroll
@@ -922,7 +963,7 @@ __global__ void __launch_bounds__(256) observe_kernel(const StepArgs a)
             }
         }
         fetch(min(y + 1, y_end - 1));  // in flight during this row's sums and shuffles
-        observe_row<VEC>(g, valid, obs, dp->rowp + (size_t)sx * ny + y, lane);
+        observe_row<VEC>(g, valid, obs, dp->colp + (size_t)sy * nx + x0, dp->rowp + (size_t)sx * ny + y, lane);
     }
     observe_flush<VEC>(dp->colp, dp->scal, nx, s, sy, x0, valid, obs, lane);
 }

@@ -322,7 +322,7 @@ __global__ void __maxnreg__(staged_max_regs<VEC>()) step_staged_kernel_q7(const 
 #pragma unroll
                 for (int j = 0; j < VEC; ++j)
                     g[i][j] = Store<ST>::get(Store<ST>::put(out[i][j], sh.q7(i)), sh.q7(i));
-            observe_row7<VEC>(g, valid, obs, rowp + y, lane);
+            observe_row7<VEC>(g, valid, obs, dp->colp + (size_t)sy * nx + x0, rowp + y, lane);
         }
         if constexpr (MIPS) {
 #pragma unroll

@@ -492,7 +492,7 @@ __global__ void __maxnreg__(staged_max_regs<VEC>()) step_staged_kernel(const Ste
 #pragma unroll
                 for (int j = 0; j < VEC; ++j)
                     g[i][j] = Store<ST>::get(Store<ST>::put(out[i][j], sh.q9(i)), sh.q9(i));
-            observe_row<VEC>(g, valid, obs, dp->rowp + (size_t)sx * ny + y, lane);
+            observe_row<VEC>(g, valid, obs, dp->colp + (size_t)sy * nx + x0, dp->rowp + (size_t)sx * ny + y, lane);
         }
         if constexpr (MIPS) {
 #pragma unroll
