@@ -16,7 +16,7 @@
  *    allocates the state and scratch buffers whose sizes lbm_buffer_bytes
  *    reports and hands them over with lbm_bind.  The context owns only host
  *    descriptors, tuning results, cached CUDA graphs, 128 bytes of pinned host
- *    memory (from the first lbm_observables on) and, for a batch of
+ *    memory (from the first lbm_bind on) and, for a batch of
  *    several launch groups (lattices differing in model, storage or velocity
  *    set), one auxiliary stream per extra group and their events, created on
  *    the first lbm_step; all of it is released by lbm_destroy.  Every call that launches

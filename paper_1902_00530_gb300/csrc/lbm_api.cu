@@ -784,12 +784,23 @@ lbm_status read_error_flag(lbm_ctx *c)
     return LBM_OK;
 }
 
-// The context's pinned host words (created once, freed by lbm_destroy), which
-// the finaliser writes: a record and the error word.
+// The context's pinned host words, which the finaliser writes: a record and the error
+// word.  Created by the first lbm_bind, freed by lbm_destroy.
 lbm_status ensure_pinned(lbm_ctx *c)
 {
     if (!c->pinned) CK(cudaMallocHost(reinterpret_cast<void **>(&c->pinned), 16 * sizeof(double)), "pinned host memory");
     return LBM_OK;
+}
+
+// While some thread captures a stream in the global mode, freeing host memory is refused to
+// every thread that is not in the relaxed mode, and the refusal ends the capture in
+// an error.  This memory is in no stream's use by then.
+void free_pinned(double *p)
+{
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    cudaFreeHost(p);
+    cudaThreadExchangeStreamCaptureMode(&mode);
 }
 
 // 16-bit populations cross to and from the host as FP32 that the device
@@ -1284,6 +1295,8 @@ lbm_status lbm_bind(lbm_ctx *c, void *state_dev, void *scratch_dev, void *cuda_s
     if (!state_dev || !scratch_dev) return fail(c, LBM_ERR_INVALID_ARG, "null buffer");
     if (((uintptr_t)state_dev & 255) || ((uintptr_t)scratch_dev & 255))
         return fail(c, LBM_ERR_INVALID_ARG, "buffers must be 256-byte aligned");
+    const lbm_status st = ensure_pinned(c);
+    if (st != LBM_OK) return st;
     drop_graphs(c);
     c->state = static_cast<char *>(state_dev);
     c->scratch = static_cast<char *>(scratch_dev);
@@ -1411,8 +1424,6 @@ lbm_status lbm_observables(lbm_ctx *c, int32_t lattice, lbm_obs *out)
         return fail(c, LBM_ERR_INVALID_ARG, "bad lattice index or null output");
     for (const GroupHost &g : c->groups) CK(launch_group_observe(c, g, c->parity), "launch observe kernel");
     // the finaliser writes the record and the error word to the pinned words
-    st = ensure_pinned(c);
-    if (st != LBM_OK) return st;
     CK(launch_finalize(all_desc(c), (int)c->lats.size(), c->max_chunk, t_dev(c), 0, 0, err_dev(c), lattice, c->pinned,
                        c->stream),
        "launch finaliser");
@@ -1835,7 +1846,7 @@ void lbm_destroy(lbm_ctx *c)
     for (cudaEvent_t e : c->ev_pool) cudaEventDestroy(e);
     for (cudaEvent_t e : c->aux_ev) cudaEventDestroy(e);
     for (cudaStream_t s : c->aux) cudaStreamDestroy(s);
-    if (c->pinned) cudaFreeHost(c->pinned);
+    if (c->pinned) free_pinned(c->pinned);
     delete c;
 }
 
