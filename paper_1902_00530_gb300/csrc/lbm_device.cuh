@@ -304,15 +304,24 @@ template <> struct VecWord<8> { using T = uint2; };
 template <> struct VecWord<16> { using T = uint4; };
 template <> struct VecWord<32> { using T = uint4; };  // two 16-byte words
 
+// A word of populations.  RO: by the read-only path (ld.global.nc), for data that no
+// thread writes while the kernel runs.  The persistent launch reads what other blocks of the
+// same launch wrote a step before, so it takes ordinary loads.
+template <bool RO, typename W> __device__ __forceinline__ W load_word(const W *p)
+{
+    if constexpr (RO) return __ldg(p);
+    else return *p;
+}
+
 // Load VEC consecutive values (aligned to VEC elements) and expand to FP32.
-template <int ST, int VEC>
+template <int ST, int VEC, bool RO>
 __device__ __forceinline__ void load_vec(const typename Store<ST>::T *p, float shift, float out[VEC])
 {
     using T = typename Store<ST>::T;
     constexpr int BYTES = (int)sizeof(T) * VEC;
     if constexpr (BYTES <= 16) {
         using W = typename VecWord<BYTES>::T;
-        W w = __ldg(reinterpret_cast<const W *>(p));
+        W w = load_word<RO>(reinterpret_cast<const W *>(p));
         if constexpr (sizeof(T) == 2 && VEC % 2 == 0) {
             unpack_words<ST, VEC>(reinterpret_cast<const uint32_t *>(&w), shift, out);
         } else {
@@ -324,7 +333,7 @@ __device__ __forceinline__ void load_vec(const typename Store<ST>::T *p, float s
         const uint4 *q = reinterpret_cast<const uint4 *>(p);
 #pragma unroll
         for (int h = 0; h < BYTES / 16; ++h) {
-            uint4 w = __ldg(q + h);
+            uint4 w = load_word<RO>(q + h);
             constexpr int PER = 16 / (int)sizeof(T);
             if constexpr (sizeof(T) == 2) {
                 unpack_words<ST, PER>(reinterpret_cast<const uint32_t *>(&w), shift, out + h * PER);
@@ -420,18 +429,27 @@ __device__ __forceinline__ float load_one(const typename Store<ST>::T *p, float 
 // Programmatic dependent launch.  Consecutive steps are dependent launches, and
 // between two plain ones the GPU idles for about a microsecond: the end of the last
 // block, the signal, the next grid's launch.  A kernel launched by
-// launch_dependent may be put on the SMs while the one before it in the stream
-// still runs (from when all of that one's blocks have called
-// allow_dependents); wait_for_previous then holds its blocks until the one before
+// launch_dependent is made ready while the one before it in the stream
+// still runs, and is put on the SMs once all of that one's blocks have ended or have called
+// allow_dependents; wait_for_previous then holds its blocks until the one before
 // has finished and its stores are visible, so a step still sees whole steps only.
 // Each kernel launched this way calls wait_for_previous before its first access to
 // what another launch writes (the descriptors are not: the host writes them between
 // launches), and some warp of every grid does, so that the waits of a chain of
-// launches imply one another.  The step kernels call allow_dependents when a block is
-// done: called at their start, waiting blocks of the next step, and of the one after,
-// fill the free warp slots unevenly and keep that imbalance when they run (720 x 240
-// D2Q7 CIL: 3.95 us per step at the end, 3.98 after the wait, 5.39 before it; 1024^2
-// CIL 14.7, 15.0, 15.1).
+// launches imply one another.
+//
+// A step kernel calls allow_dependents, if at all, after a thread's last store.  So no
+// thread stores populations while a kernel that reads them lives, which the
+// read-only loads of the latter (load_word) ask for: that call may not move up.
+//
+// The D2Q9 row-end forms read their descriptor before they wait and call it at the end
+// (1021 x 777 passive BF16: 7.3 us per step, against 7.5 if they waited first and left
+// it out).  The others wait first and leave it out: descriptor and call cost every
+// one of them registers (4096^2, us per step with and without: D2Q7 CIL FP32, vectors of 4,
+// 187 and 166, a block less per SM; passive FP16, sigma 0, 140 and 121; CIL FP16
+// 214 and 205, spills), at the price of 0.12 us per step of a launch of a few us (720 x 240
+// CIL 4.17 -> 4.29).  Called after the wait it would gain 2 % at 1024^2 CIL and lose up
+// to 8 % at 4096^2, where waiting blocks take warp slots unevenly.
 __device__ __forceinline__ void allow_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

@@ -28,7 +28,7 @@ namespace lbm {
 // Elements are addressed by their unsigned 32-bit index from the state base
 // (i plane + row pitch + x): one wide multiply-add per address.  The host
 // launches these kernels only on lattices whose q ny pitch elements fit.
-template <int ST, int VEC, int I>
+template <int ST, int VEC, int I, bool RO>
 __device__ __forceinline__ void pull_pop(const typename Store<ST>::T *base, uint32_t plane, int y, int ny,
                                          int nx, int pitch, int x0, bool valid, bool last,
                                          int lane, float shift, float out[VEC])
@@ -36,7 +36,7 @@ __device__ __forceinline__ void pull_pop(const typename Store<ST>::T *base, uint
     const uint32_t row = (uint32_t)I * plane + (uint32_t)wrap_once(y - vy(I), ny) * (uint32_t)pitch;
     float a[VEC];
     if (valid) {
-        load_vec<ST, VEC>(base + (row + (uint32_t)x0), shift, a);
+        load_vec<ST, VEC, RO>(base + (row + (uint32_t)x0), shift, a);
     } else {
 #pragma unroll
         for (int j = 0; j < VEC; ++j) a[j] = 0.f;
@@ -60,25 +60,25 @@ __device__ __forceinline__ void pull_pop(const typename Store<ST>::T *base, uint
 }
 
 // All nine populations of row y.
-template <int ST, int VEC>
+template <int ST, int VEC, bool RO>
 __device__ __forceinline__ void pull_row(const typename Store<ST>::T *base, uint32_t plane, int y,
                                          int ny, int nx, int pitch, int x0, bool valid, bool last,
                                          int lane, const Shift3 &sh, float f[9][VEC])
 {
-    pull_pop<ST, VEC, 0>(base, plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q9(0), f[0]);
-    pull_pop<ST, VEC, 1>(base, plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q9(1), f[1]);
-    pull_pop<ST, VEC, 2>(base, plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q9(2), f[2]);
-    pull_pop<ST, VEC, 3>(base, plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q9(3), f[3]);
-    pull_pop<ST, VEC, 4>(base, plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q9(4), f[4]);
-    pull_pop<ST, VEC, 5>(base, plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q9(5), f[5]);
-    pull_pop<ST, VEC, 6>(base, plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q9(6), f[6]);
-    pull_pop<ST, VEC, 7>(base, plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q9(7), f[7]);
-    pull_pop<ST, VEC, 8>(base, plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q9(8), f[8]);
+    pull_pop<ST, VEC, 0, RO>(base, plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q9(0), f[0]);
+    pull_pop<ST, VEC, 1, RO>(base, plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q9(1), f[1]);
+    pull_pop<ST, VEC, 2, RO>(base, plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q9(2), f[2]);
+    pull_pop<ST, VEC, 3, RO>(base, plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q9(3), f[3]);
+    pull_pop<ST, VEC, 4, RO>(base, plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q9(4), f[4]);
+    pull_pop<ST, VEC, 5, RO>(base, plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q9(5), f[5]);
+    pull_pop<ST, VEC, 6, RO>(base, plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q9(6), f[6]);
+    pull_pop<ST, VEC, 7, RO>(base, plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q9(7), f[7]);
+    pull_pop<ST, VEC, 8, RO>(base, plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q9(8), f[8]);
 }
 
 // The same with 64-bit pointer steps from a per-population plane pointer:
 // the copy-bound noise-free kernels, where the 32-bit form costs registers.
-template <int ST, int VEC, int I>
+template <int ST, int VEC, int I, bool RO>
 __device__ __forceinline__ void pull_pop_wide(const typename Store<ST>::T *plane, int y, int ny,
                                               int nx, int pitch, int x0, bool valid, bool last,
                                               int lane, float shift, float out[VEC])
@@ -87,7 +87,7 @@ __device__ __forceinline__ void pull_pop_wide(const typename Store<ST>::T *plane
     const typename Store<ST>::T *row = plane + (size_t)r * pitch;
     float a[VEC];
     if (valid) {
-        load_vec<ST, VEC>(row + x0, shift, a);
+        load_vec<ST, VEC, RO>(row + x0, shift, a);
     } else {
 #pragma unroll
         for (int j = 0; j < VEC; ++j) a[j] = 0.f;
@@ -110,20 +110,20 @@ __device__ __forceinline__ void pull_pop_wide(const typename Store<ST>::T *plane
     }
 }
 
-template <int ST, int VEC>
+template <int ST, int VEC, bool RO>
 __device__ __forceinline__ void pull_row_wide(const typename Store<ST>::T *base, size_t plane, int y,
                                               int ny, int nx, int pitch, int x0, bool valid, bool last,
                                               int lane, const Shift3 &sh, float f[9][VEC])
 {
-    pull_pop_wide<ST, VEC, 0>(base + 0 * plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q9(0), f[0]);
-    pull_pop_wide<ST, VEC, 1>(base + 1 * plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q9(1), f[1]);
-    pull_pop_wide<ST, VEC, 2>(base + 2 * plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q9(2), f[2]);
-    pull_pop_wide<ST, VEC, 3>(base + 3 * plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q9(3), f[3]);
-    pull_pop_wide<ST, VEC, 4>(base + 4 * plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q9(4), f[4]);
-    pull_pop_wide<ST, VEC, 5>(base + 5 * plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q9(5), f[5]);
-    pull_pop_wide<ST, VEC, 6>(base + 6 * plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q9(6), f[6]);
-    pull_pop_wide<ST, VEC, 7>(base + 7 * plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q9(7), f[7]);
-    pull_pop_wide<ST, VEC, 8>(base + 8 * plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q9(8), f[8]);
+    pull_pop_wide<ST, VEC, 0, RO>(base + 0 * plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q9(0), f[0]);
+    pull_pop_wide<ST, VEC, 1, RO>(base + 1 * plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q9(1), f[1]);
+    pull_pop_wide<ST, VEC, 2, RO>(base + 2 * plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q9(2), f[2]);
+    pull_pop_wide<ST, VEC, 3, RO>(base + 3 * plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q9(3), f[3]);
+    pull_pop_wide<ST, VEC, 4, RO>(base + 4 * plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q9(4), f[4]);
+    pull_pop_wide<ST, VEC, 5, RO>(base + 5 * plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q9(5), f[5]);
+    pull_pop_wide<ST, VEC, 6, RO>(base + 6 * plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q9(6), f[6]);
+    pull_pop_wide<ST, VEC, 7, RO>(base + 7 * plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q9(7), f[7]);
+    pull_pop_wide<ST, VEC, 8, RO>(base + 8 * plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q9(8), f[8]);
 }
 
 // A row whose length is no multiple of VEC ends inside one lane's vector: its
@@ -779,11 +779,10 @@ template <int MODEL, int ST, int VEC, bool SAMPLE> constexpr int direct_min_bloc
 // shared by the per-step launch and the persistent launch.  RAGGED: VEC need not
 // divide nx (see wrap_partial; a form of its own, since the test for it in every
 // row cost the others 5 to 9 %: 1024^2 CIL 14.3 -> 15.1 us, MIPS 21.9 -> 24.6).
-// time() gives the step's time, and is called before the first access to
-// anything another launch writes: the per-step launch waits there for the one
-// before it, having read its lattice's descriptor meanwhile (the buffers'
+// RO: populations by read-only loads (load_word).  time() gives the step's time, and is
+// called before the first access to anything another launch writes (the buffers'
 // addresses are read after it, so no load of theirs can be moved ahead of it).
-template <int MODEL, int ST, int VEC, bool SAMPLE, int NOISE, bool RAGGED = false, typename Time>
+template <int MODEL, int ST, int VEC, bool SAMPLE, int NOISE, bool RAGGED, bool RO, typename Time>
 __device__ __forceinline__ void direct_strip(const StepArgs &a, const LatDesc *dp, int s, int src_buf, Time time)
 {
     using T = typename Store<ST>::T;
@@ -820,10 +819,10 @@ __device__ __forceinline__ void direct_strip(const StepArgs &a, const LatDesc *d
     if constexpr (MODEL == MODEL_MIPS) {
         float tmp[9][VEC];
         const int yp = wrap_once(y_begin - 1, ny);
-        pull_row<ST, VEC>(src, plane32, yp, ny, nx, pitch, x0, valid, last, lane, sh, tmp);
+        pull_row<ST, VEC, RO>(src, plane32, yp, ny, nx, pitch, x0, valid, last, lane, sh, tmp);
         if (partial) wrap_partial<ST, VEC>(src, plane, yp, ny, pitch, nx - x0, sh, tmp);
         density_window<ST, VEC, RAGGED>(tmp, src, plane32, yp, nx, ny, pitch, x0, valid, last, lane, sh, rm);
-        pull_row<ST, VEC>(src, plane32, y_begin, ny, nx, pitch, x0, valid, last, lane, sh, tmp);
+        pull_row<ST, VEC, RO>(src, plane32, y_begin, ny, nx, pitch, x0, valid, last, lane, sh, tmp);
         if (partial) wrap_partial<ST, VEC>(src, plane, y_begin, ny, pitch, nx - x0, sh, tmp);
         density_window<ST, VEC, RAGGED>(tmp, src, plane32, y_begin, nx, ny, pitch, x0, valid, last, lane, sh, rc);
     }
@@ -845,14 +844,14 @@ __device__ __forceinline__ void direct_strip(const StepArgs &a, const LatDesc *d
         if constexpr (MODEL == MODEL_MIPS) {
             float fn[9][VEC];
             const int yn = wrap_once(y + 1, ny);
-            pull_row<ST, VEC>(src, plane32, yn, ny, nx, pitch, x0, valid, last, lane, sh, fn);
+            pull_row<ST, VEC, RO>(src, plane32, yn, ny, nx, pitch, x0, valid, last, lane, sh, fn);
             if (partial) wrap_partial<ST, VEC>(src, plane, yn, ny, pitch, nx - x0, sh, fn);
             density_window<ST, VEC, RAGGED>(fn, src, plane32, yn, nx, ny, pitch, x0, valid, last, lane, sh, rn);
         }
         if constexpr (WIDE)
-            pull_row_wide<ST, VEC>(src, plane, y, ny, nx, pitch, x0, valid, last, lane, sh, fc);
+            pull_row_wide<ST, VEC, RO>(src, plane, y, ny, nx, pitch, x0, valid, last, lane, sh, fc);
         else
-            pull_row<ST, VEC>(src, plane32, y, ny, nx, pitch, x0, valid, last, lane, sh, fc);
+            pull_row<ST, VEC, RO>(src, plane32, y, ny, nx, pitch, x0, valid, last, lane, sh, fc);
         if (partial) wrap_partial<ST, VEC>(src, plane, y, ny, pitch, nx - x0, sh, fc);
         float gx[VEC], gy[VEC];
         if constexpr (MODEL == MODEL_MIPS) {
@@ -901,14 +900,15 @@ __device__ __forceinline__ void direct_strip(const StepArgs &a, const LatDesc *d
 template <int MODEL, int ST, int VEC, bool SAMPLE, int NOISE, bool RAGGED>
 __global__ void __launch_bounds__(256, direct_min_blocks<MODEL, ST, VEC, SAMPLE>()) step_kernel(const StepArgs a)
 {
+    if constexpr (!RAGGED) wait_for_previous();  // see launch_dependent
     const LatDesc *dp = a.desc + find_lattice(a.desc, a.nlat, blockIdx.x);
     const int s = (blockIdx.x - dp->block_begin) * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (s >= dp->nsx * dp->nsy) return;  // whole warp leaves together
-    direct_strip<MODEL, ST, VEC, SAMPLE, NOISE, RAGGED>(a, dp, s, a.src, [&] {
-        wait_for_previous();
+    direct_strip<MODEL, ST, VEC, SAMPLE, NOISE, RAGGED, true>(a, dp, s, a.src, [&] {
+        if constexpr (RAGGED) wait_for_previous();
         return *a.t_ptr + a.k;
     });
-    allow_dependents();
+    if constexpr (RAGGED) allow_dependents();
 }
 
 // Observable partials of the stored state without stepping (same strip

@@ -118,7 +118,7 @@ template <> struct PersistStrip<9> {
     template <int MODEL, int ST, int VEC, int NOISE>
     static __device__ __forceinline__ void run(const StepArgs &a, const LatDesc *dp, int s, int src, uint32_t t)
     {
-        direct_strip<MODEL, ST, VEC, false, NOISE>(a, dp, s, src, [t] { return t; });
+        direct_strip<MODEL, ST, VEC, false, NOISE, false, false>(a, dp, s, src, [t] { return t; });
     }
 };
 

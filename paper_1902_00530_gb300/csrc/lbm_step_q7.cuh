@@ -37,7 +37,7 @@ __host__ __device__ constexpr int q7_src_dx(int i, int P)
 }
 
 // Pull row y (parity P) of population I for this lane's VEC sites.
-template <int ST, int VEC, int I, int P>
+template <int ST, int VEC, int I, int P, bool RO>
 __device__ __forceinline__ void pull_pop7(const typename Store<ST>::T *plane, int y, int ny, int nx, int pitch,
                                           int x0, bool valid, bool last, int lane, float shift, float out[VEC])
 {
@@ -45,7 +45,7 @@ __device__ __forceinline__ void pull_pop7(const typename Store<ST>::T *plane, in
     const typename Store<ST>::T *row = plane + (size_t)r * pitch;
     float a[VEC];
     if (valid) {
-        load_vec<ST, VEC>(row + x0, shift, a);
+        load_vec<ST, VEC, RO>(row + x0, shift, a);
     } else {
 #pragma unroll
         for (int j = 0; j < VEC; ++j) a[j] = 0.f;
@@ -69,18 +69,18 @@ __device__ __forceinline__ void pull_pop7(const typename Store<ST>::T *plane, in
     }
 }
 
-template <int ST, int VEC, int P>
+template <int ST, int VEC, int P, bool RO>
 __device__ __forceinline__ void pull_row7(const typename Store<ST>::T *base, size_t plane, int y, int ny, int nx,
                                           int pitch, int x0, bool valid, bool last, int lane, const Shift3 &sh,
                                           float f[7][VEC])
 {
-    pull_pop7<ST, VEC, 0, P>(base + 0 * plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q7(0), f[0]);
-    pull_pop7<ST, VEC, 1, P>(base + 1 * plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q7(1), f[1]);
-    pull_pop7<ST, VEC, 2, P>(base + 2 * plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q7(2), f[2]);
-    pull_pop7<ST, VEC, 3, P>(base + 3 * plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q7(3), f[3]);
-    pull_pop7<ST, VEC, 4, P>(base + 4 * plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q7(4), f[4]);
-    pull_pop7<ST, VEC, 5, P>(base + 5 * plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q7(5), f[5]);
-    pull_pop7<ST, VEC, 6, P>(base + 6 * plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q7(6), f[6]);
+    pull_pop7<ST, VEC, 0, P, RO>(base + 0 * plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q7(0), f[0]);
+    pull_pop7<ST, VEC, 1, P, RO>(base + 1 * plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q7(1), f[1]);
+    pull_pop7<ST, VEC, 2, P, RO>(base + 2 * plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q7(2), f[2]);
+    pull_pop7<ST, VEC, 3, P, RO>(base + 3 * plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q7(3), f[3]);
+    pull_pop7<ST, VEC, 4, P, RO>(base + 4 * plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q7(4), f[4]);
+    pull_pop7<ST, VEC, 5, P, RO>(base + 5 * plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q7(5), f[5]);
+    pull_pop7<ST, VEC, 6, P, RO>(base + 6 * plane, y, ny, nx, pitch, x0, valid, last, lane, sh.q7(6), f[6]);
 }
 
 // See wrap_partial: the populations pulled from x + 1 of a row of parity P.
@@ -267,7 +267,7 @@ struct Q7Walk {
     ObserveSums<VEC> obs;
 };
 
-template <int MODEL, int ST, int VEC, bool SAMPLE, int P, bool RAGGED>
+template <int MODEL, int ST, int VEC, bool SAMPLE, int P, bool RAGGED, bool RO>
 __device__ __forceinline__ void q7_row(Q7Walk<VEC> &w, int y, const typename Store<ST>::T *src,
                                        typename Store<ST>::T *dst, size_t plane, int nx, int ny, int pitch, int x0,
                                        bool valid, bool last, int lane, const Shift3 &sh, const SiteParams &d, bool noise,
@@ -277,11 +277,11 @@ __device__ __forceinline__ void q7_row(Q7Walk<VEC> &w, int y, const typename Sto
     const bool partial = RAGGED && valid && x0 + VEC > nx;
     if constexpr (MODEL == MODEL_MIPS) {
         const int yn = wrap_once(y + 1, ny);
-        pull_row7<ST, VEC, 1 - P>(src, plane, yn, ny, nx, pitch, x0, valid, last, lane, sh, fn);
+        pull_row7<ST, VEC, 1 - P, RO>(src, plane, yn, ny, nx, pitch, x0, valid, last, lane, sh, fn);
         if (partial) wrap_partial7<ST, VEC, 1 - P>(src, plane, yn, ny, pitch, nx - x0, sh, fn);
         density_window7<ST, VEC, 1 - P, RAGGED>(fn, src, plane, yn, nx, ny, pitch, x0, valid, last, lane, sh, w.rn);
     } else {
-        pull_row7<ST, VEC, P>(src, plane, y, ny, nx, pitch, x0, valid, last, lane, sh, w.fc);
+        pull_row7<ST, VEC, P, RO>(src, plane, y, ny, nx, pitch, x0, valid, last, lane, sh, w.fc);
         if (partial) wrap_partial7<ST, VEC, P>(src, plane, y, ny, pitch, nx - x0, sh, w.fc);
     }
     float gx[VEC], gy[VEC];
@@ -333,7 +333,7 @@ __device__ __forceinline__ void q7_row(Q7Walk<VEC> &w, int y, const typename Sto
 // read from buffer `src` and written to the other: the body of the direct
 // D2Q7 kernel, shared by the per-step launch and the persistent launch.
 // time() as in direct_strip.
-template <int MODEL, int ST, int VEC, bool SAMPLE, int NOISE, bool RAGGED = false, typename Time>
+template <int MODEL, int ST, int VEC, bool SAMPLE, int NOISE, bool RAGGED, bool RO, typename Time>
 __device__ __forceinline__ void direct_strip_q7(const StepArgs &a, const LatDesc *dp, int s, int src_buf, Time time)
 {
     using T = typename Store<ST>::T;
@@ -362,17 +362,17 @@ __device__ __forceinline__ void direct_strip_q7(const StepArgs &a, const LatDesc
         const bool partial = RAGGED && valid && x0 + VEC > nx;
         float tmp[7][VEC];
         const int yp = wrap_once(y_begin - 1, ny);  // odd
-        pull_row7<ST, VEC, 1>(src, plane, yp, ny, nx, pitch, x0, valid, last, lane, sh, tmp);
+        pull_row7<ST, VEC, 1, RO>(src, plane, yp, ny, nx, pitch, x0, valid, last, lane, sh, tmp);
         if (partial) wrap_partial7<ST, VEC, 1>(src, plane, yp, ny, pitch, nx - x0, sh, tmp);
         density_window7<ST, VEC, 1, RAGGED>(tmp, src, plane, yp, nx, ny, pitch, x0, valid, last, lane, sh, w.rm);
-        pull_row7<ST, VEC, 0>(src, plane, y_begin, ny, nx, pitch, x0, valid, last, lane, sh, w.fc);
+        pull_row7<ST, VEC, 0, RO>(src, plane, y_begin, ny, nx, pitch, x0, valid, last, lane, sh, w.fc);
         if (partial) wrap_partial7<ST, VEC, 0>(src, plane, y_begin, ny, pitch, nx - x0, sh, w.fc);
         density_window7<ST, VEC, 0, RAGGED>(w.fc, src, plane, y_begin, nx, ny, pitch, x0, valid, last, lane, sh, w.rc);
     }
     for (int y = y_begin; y < y_end; y += 2) {
-        q7_row<MODEL, ST, VEC, SAMPLE, 0, RAGGED>(w, y, src, dst, plane, nx, ny, pitch, x0, valid, last, lane, sh, d, noise,
+        q7_row<MODEL, ST, VEC, SAMPLE, 0, RAGGED, RO>(w, y, src, dst, plane, nx, ny, pitch, x0, valid, last, lane, sh, d, noise,
                                           t, id, a.rk, colp, rowp);
-        q7_row<MODEL, ST, VEC, SAMPLE, 1, RAGGED>(w, y + 1, src, dst, plane, nx, ny, pitch, x0, valid, last, lane, sh, d,
+        q7_row<MODEL, ST, VEC, SAMPLE, 1, RAGGED, RO>(w, y + 1, src, dst, plane, nx, ny, pitch, x0, valid, last, lane, sh, d,
                                           noise, t, id, a.rk, colp, rowp);
     }
     if constexpr (SAMPLE) observe_flush<VEC>(dp->colp, dp->scal, nx, s, sy, x0, valid, w.obs, lane);
@@ -381,14 +381,11 @@ __device__ __forceinline__ void direct_strip_q7(const StepArgs &a, const LatDesc
 template <int MODEL, int ST, int VEC, bool SAMPLE, int NOISE, bool RAGGED>
 __global__ void __launch_bounds__(256) step_kernel_q7(const StepArgs a)
 {
+    wait_for_previous();  // see launch_dependent
     const LatDesc *dp = a.desc + find_lattice(a.desc, a.nlat, blockIdx.x);
     const int s = (blockIdx.x - dp->block_begin) * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (s >= dp->nsx * dp->nsy) return;  // whole warp leaves together
-    direct_strip_q7<MODEL, ST, VEC, SAMPLE, NOISE, RAGGED>(a, dp, s, a.src, [&] {
-        wait_for_previous();
-        return *a.t_ptr + a.k;
-    });
-    allow_dependents();
+    direct_strip_q7<MODEL, ST, VEC, SAMPLE, NOISE, RAGGED, true>(a, dp, s, a.src, [&] { return *a.t_ptr + a.k; });
 }
 
 // The D2Q7 strip update of the persistent launch (lbm_step_persistent.cuh).
@@ -396,7 +393,7 @@ template <> struct PersistStrip<7> {
     template <int MODEL, int ST, int VEC, int NOISE>
     static __device__ __forceinline__ void run(const StepArgs &a, const LatDesc *dp, int s, int src, uint32_t t)
     {
-        direct_strip_q7<MODEL, ST, VEC, false, NOISE>(a, dp, s, src, [t] { return t; });
+        direct_strip_q7<MODEL, ST, VEC, false, NOISE, false, false>(a, dp, s, src, [t] { return t; });
     }
 };
 
