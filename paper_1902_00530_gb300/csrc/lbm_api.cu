@@ -469,7 +469,6 @@ StepArgs step_args(const lbm_ctx *c, const GroupHost &g, int src, uint32_t k)
     a.key0 = (uint32_t)c->seed;
     a.key1 = (uint32_t)(c->seed >> 32);
     a.stages = g.stages;
-    a.ragged = 0;
     a.err = err_dev(c);
     for (int r = 0; r < 10; ++r) {  // Philox round keys (Weyl increments, Salmon et al. 2011)
         a.rk[2 * r] = a.key0 + (uint32_t)r * 0x9E3779B9u;
@@ -497,7 +496,8 @@ cudaError_t launch_group_step(const lbm_ctx *c, const GroupHost &g, int src, uin
         a.desc = reinterpret_cast<const LatDesc *>(c->scratch + g.plain_off);
         a.stages = kind = 0;
         vec = g.plain.vec;
-        for (int m : g.members) a.ragged |= c->lats[m].lat.nx % vec != 0;
+        for (int m : g.members)
+            if (c->lats[m].lat.nx % vec) kind = 2;
         blocks = g.plain_blocks;
         warps = g.plain.warps;
     }
@@ -606,7 +606,6 @@ cudaError_t launch_group_observe(const lbm_ctx *c, const GroupHost &g, int src)
     a.t_ptr = t_dev(c);
     a.k = 0;
     a.key0 = a.key1 = 0;
-    a.ragged = 0;
     a.stages = g.stages;  // the strip-to-block mapping follows the group's step kernel
     a.err = err_dev(c);
     for (int r = 0; r < 20; ++r) a.rk[r] = 0;

@@ -139,10 +139,22 @@ struct StepArgs {
     uint32_t k;           // step offset of this launch from *t_ptr
     uint32_t key0, key1;  // Philox key = seed
     int stages;           // staged kernel: shared-memory row buffers per warp
-    int ragged;           // direct kernel: the vector width need not divide nx
     unsigned *err;        // device error word (bounded waits report here)
     uint32_t rk[20];      // Philox round keys: (key0 + r W0, key1 + r W1), r = 0..9
 };
+
+// The round keys are read as kernel parameters, four at a time where they lie at a
+// multiple of 16 bytes (as above), else in pairs.  The direct kernels need the former: with
+// one more word before them step_kernel<CIL, F32, 4, noise> spilled 32 bytes of its 80
+// registers where it spills none, the F16 form 100 for 68.  The staged and the persistent
+// kernels, which hold more besides, need the latter (bytes spilled with fours and with
+// pairs: persistent D2Q9 CIL F32, vectors of 4, 4 and 0, D2Q7 8 and 0; staged CIL F16,
+// vectors of 8, 88 and 32).  They take their arguments in this form.
+struct StepArgsPairs {
+    int at_8_bytes[2];
+    StepArgs a;
+};
+static_assert(offsetof(StepArgs, rk) % 16 == 0 && offsetof(StepArgsPairs, a) % 16 == 8, "see above");
 
 // The persistent launch's work list (lbm_step_persistent.cuh): items are the
 // blocks of the per-step grid, one per step, taken in order by a counter.
@@ -438,18 +450,17 @@ __device__ __forceinline__ float load_one(const typename Store<ST>::T *p, float 
 // launches), and some warp of every grid does, so that the waits of a chain of
 // launches imply one another.
 //
-// A step kernel calls allow_dependents, if at all, after a thread's last store.  So no
-// thread stores populations while a kernel that reads them lives, which the
-// read-only loads of the latter (load_word) ask for: that call may not move up.
+// A step kernel calls allow_dependents in the last pass of its row loop, after the
+// thread's last stores.  So no thread stores populations while a kernel that reads them lives,
+// which the read-only loads of the latter (load_word) ask for: that call may not move
+// up.  Behind the loop it cost every one of the kernels registers (4096^2, us per step there
+// and here: D2Q7 CIL FP32, vectors of 4, 187 and 166, a block more per SM; passive FP16,
+// sigma 0, 140 and 121; CIL FP16 214 and 205, spills); in the loop it costs none.
 //
-// The D2Q9 row-end forms read their descriptor before they wait and call it at the end
-// (1021 x 777 passive BF16: 7.3 us per step, against 7.5 if they waited first and left
-// it out).  The others wait first and leave it out: descriptor and call cost every
-// one of them registers (4096^2, us per step with and without: D2Q7 CIL FP32, vectors of 4,
-// 187 and 166, a block less per SM; passive FP16, sigma 0, 140 and 121; CIL FP16
-// 214 and 205, spills), at the price of 0.12 us per step of a launch of a few us (720 x 240
-// CIL 4.17 -> 4.29).  Called after the wait it would gain 2 % at 1024^2 CIL and lose up
-// to 8 % at 4096^2, where waiting blocks take warp slots unevenly.
+// The descriptor is read before the wait where the registers allow: D2Q7 with up to four
+// sites per lane (720 x 240 CIL 4.02 us per step, 4.28 waiting first) and the D2Q9
+// row-end forms (1021 x 777 passive BF16 7.2, 7.5).  The other D2Q9 forms wait first: held
+// over the wait it makes step_kernel<CIL, F32, 4, noise> spill 28 bytes of its 80 registers.
 __device__ __forceinline__ void allow_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

@@ -893,6 +893,7 @@ __device__ __forceinline__ void direct_strip(const StepArgs &a, const LatDesc *d
                 rc[j] = rn[j];
             }
         }
+        if (!SAMPLE && RO && y + 1 == y_end) allow_dependents();
     }
     if constexpr (SAMPLE) observe_flush<VEC>(dp->colp, dp->scal, nx, s, sy, x0, valid, obs, lane);
 }
@@ -900,7 +901,7 @@ __device__ __forceinline__ void direct_strip(const StepArgs &a, const LatDesc *d
 template <int MODEL, int ST, int VEC, bool SAMPLE, int NOISE, bool RAGGED>
 __global__ void __launch_bounds__(256, direct_min_blocks<MODEL, ST, VEC, SAMPLE>()) step_kernel(const StepArgs a)
 {
-    if constexpr (!RAGGED) wait_for_previous();  // see launch_dependent
+    if constexpr (!RAGGED) wait_for_previous();  // see allow_dependents
     const LatDesc *dp = a.desc + find_lattice(a.desc, a.nlat, blockIdx.x);
     const int s = (blockIdx.x - dp->block_begin) * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (s >= dp->nsx * dp->nsy) return;  // whole warp leaves together
@@ -908,7 +909,6 @@ __global__ void __launch_bounds__(256, direct_min_blocks<MODEL, ST, VEC, SAMPLE>
         if constexpr (RAGGED) wait_for_previous();
         return *a.t_ptr + a.k;
     });
-    if constexpr (RAGGED) allow_dependents();
 }
 
 // Observable partials of the stored state without stepping (same strip

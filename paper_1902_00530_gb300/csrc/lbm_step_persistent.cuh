@@ -109,7 +109,14 @@ __device__ __forceinline__ void persist_setup(const StepArgs &a, const PersistAr
 #ifndef LBM_PERSIST_REGS
 #define LBM_PERSIST_REGS 96
 #endif
-template <int MODEL> constexpr int persist_max_regs() { return MODEL == MODEL_MIPS ? 128 : LBM_PERSIST_REGS; }
+// The noisy D2Q7 strips of up to four sites per lane fit 80, where six blocks of 4 warps
+// share an SM and not five (4096^2 passive, us per step at 80 and at 89: BF16 152.9,
+// FP16 168).
+template <int Q, int MODEL, int VEC, int NOISE> constexpr int persist_max_regs()
+{
+    if (MODEL == MODEL_MIPS) return 128;
+    return Q == 7 && VEC <= 4 && NOISE == 1 ? 80 : LBM_PERSIST_REGS;
+}
 
 // The strip update of lattice Q (9: D2Q9, 7: D2Q7); the D2Q7 form is defined
 // beside its direct kernel.
@@ -123,8 +130,9 @@ template <> struct PersistStrip<9> {
 };
 
 template <int Q, int MODEL, int ST, int VEC, int NOISE>
-__global__ void __maxnreg__(persist_max_regs<MODEL>()) step_persistent_kernel(const StepArgs a, const PersistArgs p)
+__global__ void __maxnreg__((persist_max_regs<Q, MODEL, VEC, NOISE>())) step_persistent_kernel(const StepArgsPairs args, const PersistArgs p)
 {
+    const StepArgs &a = args.a;
     __shared__ PersistItem it;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned total = (unsigned)p.nsteps * (unsigned)p.pg[p.npg];
@@ -212,7 +220,7 @@ static cudaError_t launch_persistent_one(const StepArgs &a, const PersistArgs &p
     if (e != cudaSuccess) return e;
     const long long items = (long long)p.nsteps * step_blocks;
     const int grid = (int)std::min<long long>(items, (long long)std::max(1, per_sm) * sms);
-    kern<<<grid, warps * 32, 0, stream>>>(a, p);
+    kern<<<grid, warps * 32, 0, stream>>>(StepArgsPairs{{0, 0}, a}, p);
     return cudaGetLastError();
 }
 

@@ -374,6 +374,7 @@ __device__ __forceinline__ void direct_strip_q7(const StepArgs &a, const LatDesc
                                           t, id, a.rk, colp, rowp);
         q7_row<MODEL, ST, VEC, SAMPLE, 1, RAGGED, RO>(w, y + 1, src, dst, plane, nx, ny, pitch, x0, valid, last, lane, sh, d,
                                           noise, t, id, a.rk, colp, rowp);
+        if (!SAMPLE && RO && y + 2 >= y_end) allow_dependents();
     }
     if constexpr (SAMPLE) observe_flush<VEC>(dp->colp, dp->scal, nx, s, sy, x0, valid, w.obs, lane);
 }
@@ -381,11 +382,15 @@ __device__ __forceinline__ void direct_strip_q7(const StepArgs &a, const LatDesc
 template <int MODEL, int ST, int VEC, bool SAMPLE, int NOISE, bool RAGGED>
 __global__ void __launch_bounds__(256) step_kernel_q7(const StepArgs a)
 {
-    wait_for_previous();  // see launch_dependent
+    constexpr bool LATE = VEC <= 4;  // waits with its descriptor read: see allow_dependents
+    if constexpr (!LATE) wait_for_previous();
     const LatDesc *dp = a.desc + find_lattice(a.desc, a.nlat, blockIdx.x);
     const int s = (blockIdx.x - dp->block_begin) * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (s >= dp->nsx * dp->nsy) return;  // whole warp leaves together
-    direct_strip_q7<MODEL, ST, VEC, SAMPLE, NOISE, RAGGED, true>(a, dp, s, a.src, [&] { return *a.t_ptr + a.k; });
+    direct_strip_q7<MODEL, ST, VEC, SAMPLE, NOISE, RAGGED, true>(a, dp, s, a.src, [&] {
+        if constexpr (LATE) wait_for_previous();
+        return *a.t_ptr + a.k;
+    });
 }
 
 // The D2Q7 strip update of the persistent launch (lbm_step_persistent.cuh).

@@ -152,8 +152,9 @@ __device__ __forceinline__ void stage_density_window7(const typename Store<ST>::
 }
 
 template <int MODEL, int ST, int VEC, bool SAMPLE, int NOISE>
-__global__ void __maxnreg__(staged_max_regs<VEC>()) step_staged_kernel_q7(const StepArgs a)
+__global__ void __maxnreg__(staged_max_regs<VEC>()) step_staged_kernel_q7(const StepArgsPairs args)
 {
+    const StepArgs &a = args.a;
     using T = typename Store<ST>::T;
     using G = StageGeom7<ST, VEC>;
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -169,7 +170,7 @@ __global__ void __maxnreg__(staged_max_regs<VEC>()) step_staged_kernel_q7(const 
     uint64_t *full = reinterpret_cast<uint64_t *>(smem_raw + (size_t)S * stage_elems * sizeof(T));
     uint64_t *empty = full + S;
     float *const cv0 = reinterpret_cast<float *>(empty + S) + (size_t)warp * 7 * G::W + (threadIdx.x & 31) * VEC;
-    auto cv = [&](int q) { return cv0 + (size_t)(q & 1) * warps * 7 * G::W; };
+    auto cv = [&](int parity) { return cv0 + (size_t)parity * warps * 7 * G::W; };
 
     const StagedBlock blk = staged_block(a, warps);
     const LatDesc *dp = blk.dp;
@@ -205,7 +206,7 @@ __global__ void __maxnreg__(staged_max_regs<VEC>()) step_staged_kernel_q7(const 
     constexpr bool MIPS = (MODEL == MODEL_MIPS);
     const int q_first_row = MIPS ? y_begin - 1 : y_begin;
     const int nq = (y_end - y_begin) + (MIPS ? 2 : 0);
-    auto stage_ptr = [&](RingPos r) { return ring + (size_t)r.slot * stage_elems; };
+    auto stage_ptr = [&](RingPos r) { return ring + (size_t)r.slot() * stage_elems; };
     bool ok = true;
     auto fail = [&]() {
         ok = false;
@@ -225,17 +226,17 @@ __global__ void __maxnreg__(staged_max_regs<VEC>()) step_staged_kernel_q7(const 
     auto release = [&](RingPos r) {
         __syncwarp();
         if (blk.nact == 1) {  // a single warp: its own reads are all there is to wait for
-            if (ok && issued < nq) issue(r.slot);
+            if (ok && issued < nq) issue(r.slot());
             return;
         }
-        if (lane == 0) mbar_arrive(&empty[r.slot]);
+        if (lane == 0) mbar_arrive(&empty[r.slot()]);
         if (leader && ok && issued < nq) {
-            if (!stage_wait(&empty[r.slot], r.phase)) fail();
-            else issue(r.slot);
+            if (!stage_wait(&empty[r.slot()], r.phase())) fail();
+            else issue(r.slot());
         }
     };
     auto wait_row = [&](RingPos r) {
-        if (ok && !stage_wait(&full[r.slot], r.phase)) fail();
+        if (ok && !stage_wait(&full[r.slot()], r.phase())) fail();
         return ok;
     };
 
@@ -244,17 +245,16 @@ __global__ void __maxnreg__(staged_max_regs<VEC>()) step_staged_kernel_q7(const 
     double *rowp = dp->rowp + (size_t)sx * ny;
 
     float rm[VEC + 2], rc[VEC + 2], rn[VEC + 2];
-    int q = 0;            // row to update next, and its place in the ring
-    RingPos at{0, 0u};
+    int y_next = y_begin;  // row to update next, and its place in the ring
+    RingPos at{0};
     if constexpr (MIPS) {
         if (wait_row(at)) {
             stage_density_window7<ST, VEC, 1>(stage_ptr(at), sg, b, sh, lane, rm);  // row y_begin-1: odd
             release(at);
         }
-        q = 1;
         at = at.next(S);
         if (wait_row(at)) {
-            stage_density_window7<ST, VEC, 0>(stage_ptr(at), sg, b, sh, lane, rc, CONV ? cv(1) : nullptr, G::W);
+            stage_density_window7<ST, VEC, 0>(stage_ptr(at), sg, b, sh, lane, rc, CONV ? cv(0) : nullptr, G::W);
             if constexpr (CONV) release(at);
         }
     }
@@ -270,10 +270,10 @@ __global__ void __maxnreg__(staged_max_regs<VEC>()) step_staged_kernel_q7(const 
                 at = cur;
                 return false;
             }
-            stage_density_window7<ST, VEC, 1 - P>(stage_ptr(at), sg, b, sh, lane, rn, cv(q + 1), G::W);
+            stage_density_window7<ST, VEC, 1 - P>(stage_ptr(at), sg, b, sh, lane, rn, cv(1 - P), G::W);
             release(at);
 #pragma unroll
-            for (int i = 0; i < 7; ++i) get_f32<VEC>(cv(q) + i * G::W, f[i]);
+            for (int i = 0; i < 7; ++i) get_f32<VEC>(cv(P) + i * G::W, f[i]);
         } else if constexpr (MIPS) {
             if (!wait_row(at)) {
                 at = cur;
@@ -290,7 +290,7 @@ __global__ void __maxnreg__(staged_max_regs<VEC>()) step_staged_kernel_q7(const 
             stage_row7<ST, VEC, P>(stage_ptr(cur), sg, b, sh, f);
             release(cur);
         }
-        ++q;
+        y_next = y + 1;
         float gx[VEC], gy[VEC];
         if constexpr (MIPS) {
             mips_gradients7<VEC, P>(rm, rc, rn, gx, gy);
@@ -342,7 +342,7 @@ __global__ void __maxnreg__(staged_max_regs<VEC>()) step_staged_kernel_q7(const 
         // the copies warp 0 issued must land before the block's shared memory is
         // released: wait for the rows it has not waited for itself (bounded)
         RingPos r = MIPS ? at.next(S) : at;
-        for (int qq = q + (MIPS ? 1 : 0); qq < issued; ++qq, r = r.next(S)) (void)stage_wait(&full[r.slot], r.phase);
+        for (int qq = (y_next - y_begin) + (MIPS ? 2 : 0); qq < issued; ++qq, r = r.next(S)) (void)stage_wait(&full[r.slot()], r.phase());
     }
     if (!ok) return;
     if constexpr (SAMPLE) observe_flush<VEC>(dp->colp, dp->scal, nx, s, sy, x0, valid, obs, lane);
@@ -356,7 +356,7 @@ static cudaError_t launch_one_staged7(const StepArgs &a, int blocks, int warps, 
     auto kern = step_staged_kernel_q7<MODEL, ST, VEC, SAMPLE, NOISE>;
     cudaError_t e = allow_all_smem(kern);
     if (e != cudaSuccess) return e;
-    kern<<<blocks, warps * 32, bytes, stream>>>(a);
+    kern<<<blocks, warps * 32, bytes, stream>>>(StepArgsPairs{{0, 0}, a});
     return cudaGetLastError();
 }
 
@@ -369,7 +369,7 @@ static cudaError_t launch_one_q7(int kind, const StepArgs &a, int blocks, int wa
     if (kind == 1) return launch_one_staged7<MODEL, ST, VEC, SAMPLE, NOISE>(a, blocks, warps, stream);
     const dim3 grid(blocks), block(warps * 32);
     if constexpr (!SAMPLE && VEC > 1) {
-        if (a.ragged)
+        if (kind == 2)
             return launch_dependent(step_kernel_q7<MODEL, ST, VEC, SAMPLE, NOISE, true>, grid, block, 0, stream, a);
     }
     return launch_dependent(step_kernel_q7<MODEL, ST, VEC, SAMPLE, NOISE, false>, grid, block, 0, stream, a);

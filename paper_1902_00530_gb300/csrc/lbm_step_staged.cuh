@@ -292,15 +292,13 @@ template <int VEC> constexpr int staged_max_regs()
 
 // A row's place in the ring: its buffer and the phase parity of the buffer's
 // barriers.  Both advance by counting: row q's are q mod S and (q / S) mod 2, but S is
-// not a constant, and the divisions, several per row and lane, were about 25 of
-// the 326 instructions per site of the FP32 MIPS kernel.
+// not a constant, and a division is a chain of a dozen instructions.  One word, since
+// the kernels of 8-site vectors have no register to spare.
 struct RingPos {
-    int slot;
-    uint32_t phase;
-    __device__ __forceinline__ RingPos next(int S) const
-    {
-        return slot + 1 == S ? RingPos{0, phase ^ 1u} : RingPos{slot + 1, phase};
-    }
+    int v;  // 2 slot + phase
+    __device__ __forceinline__ int slot() const { return v >> 1; }
+    __device__ __forceinline__ uint32_t phase() const { return (uint32_t)v & 1u; }
+    __device__ __forceinline__ RingPos next(int S) const { return RingPos{v + 2 < 2 * S ? v + 2 : (v & 1) ^ 1}; }
 };
 
 // The block's place in its lattice: strip row sy, first strip column sx0, and
@@ -323,8 +321,9 @@ __device__ __forceinline__ StagedBlock staged_block(const StepArgs &a, int warps
 }
 
 template <int MODEL, int ST, int VEC, bool SAMPLE, int NOISE>
-__global__ void __maxnreg__(staged_max_regs<VEC>()) step_staged_kernel(const StepArgs a)
+__global__ void __maxnreg__(staged_max_regs<VEC>()) step_staged_kernel(const StepArgsPairs args)
 {
+    const StepArgs &a = args.a;
     using T = typename Store<ST>::T;
     using G = StageGeom<ST, VEC>;
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -377,7 +376,7 @@ __global__ void __maxnreg__(staged_max_regs<VEC>()) step_staged_kernel(const Ste
     constexpr bool MIPS = (MODEL == MODEL_MIPS);
     const int q_first_row = MIPS ? y_begin - 1 : y_begin;
     const int nq = (y_end - y_begin) + (MIPS ? 2 : 0);
-    auto stage_ptr = [&](RingPos r) { return ring + (size_t)r.slot * stage_elems; };
+    auto stage_ptr = [&](RingPos r) { return ring + (size_t)r.slot() * stage_elems; };
     bool ok = true;
     auto fail = [&]() {
         ok = false;
@@ -398,17 +397,17 @@ __global__ void __maxnreg__(staged_max_regs<VEC>()) step_staged_kernel(const Ste
     auto release = [&](RingPos r) {
         __syncwarp();
         if (blk.nact == 1) {  // a single warp: its own reads are all there is to wait for
-            if (ok && issued < nq) issue(r.slot);
+            if (ok && issued < nq) issue(r.slot());
             return;
         }
-        if (lane == 0) mbar_arrive(&empty[r.slot]);
+        if (lane == 0) mbar_arrive(&empty[r.slot()]);
         if (leader && ok && issued < nq) {
-            if (!stage_wait(&empty[r.slot], r.phase)) fail();
-            else issue(r.slot);
+            if (!stage_wait(&empty[r.slot()], r.phase())) fail();
+            else issue(r.slot());
         }
     };
     auto wait_row = [&](RingPos r) {
-        if (ok && !stage_wait(&full[r.slot], r.phase)) fail();
+        if (ok && !stage_wait(&full[r.slot()], r.phase())) fail();
         return ok;
     };
 
@@ -421,7 +420,7 @@ __global__ void __maxnreg__(staged_max_regs<VEC>()) step_staged_kernel(const Ste
     // released one row earlier.
     float rm[VEC + 2], rc[VEC + 2], rn[VEC + 2];
     int q = 0;            // row to update next, and its place in the ring
-    RingPos at{0, 0u};
+    RingPos at{0};
     if constexpr (MIPS) {
         if (wait_row(at)) {
             stage_density_window<ST, VEC>(stage_ptr(at), sg, b, sh, lane, rm);
@@ -507,7 +506,7 @@ __global__ void __maxnreg__(staged_max_regs<VEC>()) step_staged_kernel(const Ste
         // is released: wait for the rows it has not waited for itself (the
         // latest phase of each of their buffers; bounded)
         RingPos r = MIPS ? at.next(S) : at;
-        for (int qq = q + (MIPS ? 1 : 0); qq < issued; ++qq, r = r.next(S)) (void)stage_wait(&full[r.slot], r.phase);
+        for (int qq = q + (MIPS ? 1 : 0); qq < issued; ++qq, r = r.next(S)) (void)stage_wait(&full[r.slot()], r.phase());
     }
     if (!ok) return;
     if constexpr (SAMPLE) observe_flush<VEC>(dp->colp, dp->scal, nx, s, sy, x0, valid, obs, lane);
@@ -529,7 +528,7 @@ static cudaError_t launch_one_staged(const StepArgs &a, int blocks, int warps, c
     auto kern = step_staged_kernel<MODEL, ST, VEC, SAMPLE, NOISE>;
     cudaError_t e = allow_all_smem(kern);
     if (e != cudaSuccess) return e;
-    kern<<<blocks, warps * 32, bytes, stream>>>(a);
+    kern<<<blocks, warps * 32, bytes, stream>>>(StepArgsPairs{{0, 0}, a});
     return cudaGetLastError();
 }
 
@@ -539,7 +538,7 @@ static cudaError_t launch_one(int kind, const StepArgs &a, int blocks, int warps
     if (kind == 1) return launch_one_staged<MODEL, ST, VEC, SAMPLE, NOISE>(a, blocks, warps, stream);
     const dim3 grid(blocks), block(warps * 32);
     if constexpr (!SAMPLE && VEC > 1) {
-        if (a.ragged)
+        if (kind == 2)
             return launch_dependent(step_kernel<MODEL, ST, VEC, SAMPLE, NOISE, true>, grid, block, 0, stream, a);
     }
     return launch_dependent(step_kernel<MODEL, ST, VEC, SAMPLE, NOISE, false>, grid, block, 0, stream, a);

@@ -52,18 +52,21 @@ def test_persistent_strips_take_ordinary_loads():
 
 
 def test_per_step_kernels_wait_before_populations_and_release_after_them():
-    for name, kernel, strip in (("lbm_step.cuh", "step_kernel", "direct_strip"),
-                                ("lbm_step_q7.cuh", "step_kernel_q7", "direct_strip_q7")):
+    for name, kernel, strip, stores in (("lbm_step.cuh", "step_kernel", "direct_strip", "store_vec<"),
+                                        ("lbm_step_q7.cuh", "step_kernel_q7", "direct_strip_q7", "q7_row<")):
         src = _source(name)
         body = _body(src, r"\b" + kernel + r"\(const StepArgs a\)")
         # the wait comes first, or in time(), which the strip calls before it reads a buffer's address
         call = body[body.index(strip + "<"):]
         first = body[1:].lstrip().startswith("wait_for_previous();")
-        ragged_later = (body[1:].lstrip().startswith("if constexpr (!RAGGED) wait_for_previous();")
-                        and "if constexpr (RAGGED) wait_for_previous();" in call[:call.index("});")])
-        assert first or ragged_later, name
+        either = re.search(r"if constexpr \(!(\w+)\) wait_for_previous\(\);", body[:body.index(strip + "<")])
+        late = bool(either) and f"if constexpr ({either[1]}) wait_for_previous();" in call[:call.index("});")]
+        assert first or late, name
+        assert "allow_dependents" not in body
         update = _body(src, r"__forceinline__ void " + strip + r"\(")
         assert update.index("time()") < update.index("dp->f[")
-        # dependents only after the strip's stores
-        assert "allow_dependents" not in body[:body.index(strip + "<")] + call[:call.index(";")]
-        assert "allow_dependents" not in update
+        # dependents only after the stores of the strip's last row
+        assert update.count("allow_dependents") == 1
+        release = update.index("allow_dependents")
+        assert release > update.rindex(stores)
+        assert re.search(r"y \+ [12] (==|>=) y_end\) $", update[:release]), name
