@@ -38,9 +38,13 @@ constexpr int TUNE_STEPS_PERSIST = 12;   // ... and as one persistent launch (lo
 constexpr float TUNE_MIN_MS = 0.25f;     // shorter timings are repeated over more steps (event resolution, noise)
 constexpr int TUNE_STEPS_MAX = 256;
 // the tuner's second look: at most so many candidates within this factor of the fastest, so often
-constexpr size_t TUNE_FINALISTS = 5;
+constexpr size_t TUNE_FINALISTS = 4;
 constexpr float TUNE_FINAL_MARGIN = 1.08f;
 constexpr int TUNE_FINAL_REPS = 2;
+// plain shapes: the tallest strips tried, and how near the fastest a vector's first
+// time lies for its other heights to be tried
+constexpr int PLAIN_ROWS_MAX = 32;
+constexpr float PLAIN_NEAR = 1.15f;
 // Mode 2 considers persistent launches only for groups with at least this
 // many sites per step.  Below it a step's items cannot fill the GPU in either
 // form and the persistent launch's dependency waits cost more than a launch
@@ -1073,21 +1077,63 @@ lbm_status tune_group(lbm_ctx *c, GroupHost &g, std::vector<Choice> *alts)
     // strips, 4.5 in shorter ones.  Vectors that do not divide nx (a row then
     // ends inside a lane's vector, wrap_partial): one site per thread costs an odd
     // width up to twice the instructions per site.
+    // Not every shape is timed (four vectors, six heights and two block sizes made
+    // an odd width's tuning five times as long: 1021 x 777 BF16 20 ms, now 9, with
+    // the same choice): each vector at one height,
+    // then, for the vectors near the fastest, the heights up and down from it
+    // while they are faster, then the fastest shape in blocks of 8 warps.
     if (c->persist_mode != 1 && best_step < 1e29f && direct && !settled) {
-        for (int v : all_v) {
-            if (!allowed_vec(g.storage, v)) continue;
+        auto offered = [&](int v, int r) {
             bool divides = true;
             for (int m : g.members) divides = divides && (c->lats[m].lat.nx % v == 0);
-            for (int r : {1, 2, 4, 8, 16, 32}) {
-                if (r < ROWS_MIN ? group_sites > SHORT_STRIP_MAX_SITES : divides) continue;
-                if ((g.q == 7 && r == 1) || (r > ROWS_MIN && r > 2 * max_ny)) continue;
-                for (int w : {4, 8}) {
-                    Choice now = bstep;
-                    now.plain = {v, r, w, 0};
-                    st = consider(now, TUNE_STEPS);
+            if (r < (g.q == 7 ? 2 : 1) || r > PLAIN_ROWS_MAX || (r > ROWS_MIN && r > 2 * max_ny)) return false;
+            return r < ROWS_MIN ? group_sites <= SHORT_STRIP_MAX_SITES : !divides;
+        };
+        // times plain shape sh; *ms stays as it is where it does not run
+        auto time_plain = [&](const Shape &sh, float *ms) -> lbm_status {
+            Choice now = bstep;
+            now.plain = sh;
+            const size_t n = timed.size();
+            const lbm_status st = consider(now, TUNE_STEPS);
+            if (st == LBM_OK && timed.size() > n) *ms = timed.back().first;
+            return st;
+        };
+        const int r0 = group_sites <= SHORT_STRIP_MAX_SITES ? 4 : 16;
+        float first[4] = {1e30f, 1e30f, 1e30f, 1e30f}, fastest = 1e30f;
+        Shape win{0, 0, 0, 0};
+        auto note = [&](const Shape &sh, float ms) {
+            const bool faster = ms < fastest;
+            if (faster) fastest = ms, win = sh;
+            return faster;
+        };
+        for (int k = 0; k < 4; ++k) {
+            if (!allowed_vec(g.storage, all_v[k]) || !offered(all_v[k], r0)) continue;
+            const Shape sh{all_v[k], r0, 4, 0};
+            st = time_plain(sh, &first[k]);
+            if (st != LBM_OK) return st;
+            note(sh, first[k]);
+        }
+        const float near = PLAIN_NEAR * fastest;
+        for (int k = 0; k < 4; ++k) {
+            if (first[k] > near || first[k] > 1e29f) continue;
+            for (int up = 0; up < 2; ++up) {
+                float last = first[k];
+                for (int r = up ? 2 * r0 : r0 / 2; offered(all_v[k], r); r = up ? 2 * r : r / 2) {
+                    const Shape sh{all_v[k], r, 4, 0};
+                    float ms = 1e30f;
+                    st = time_plain(sh, &ms);
                     if (st != LBM_OK) return st;
+                    note(sh, ms);
+                    if (!(ms < last)) break;
+                    last = ms;
                 }
             }
+        }
+        if (win.rows > 0) {
+            float ms = 1e30f;
+            win.warps = 8;
+            st = time_plain(win, &ms);
+            if (st != LBM_OK) return st;
         }
     }
     if (b.plain.rows > 0) alts->push_back(bstep);
@@ -1103,8 +1149,7 @@ lbm_status tune_group(lbm_ctx *c, GroupHost &g, std::vector<Choice> *alts)
             st = upload_descs(c);
             if (st != LBM_OK) return st;
             float ms = 0.f;
-            st = time_form(resident_ok(c, g) || persistent_ok(c, g) ? TUNE_STEPS_PERSIST : TUNE_STEPS, &ms,
-                           2 * TUNE_MIN_MS);
+            st = time_form(resident_ok(c, g) || persistent_ok(c, g) ? TUNE_STEPS_PERSIST : TUNE_STEPS, &ms);
             if (st != LBM_OK) return st;
             again[k] = std::min(again[k], ms);
         }
