@@ -257,6 +257,19 @@ lbm_status lbm_tune(lbm_ctx *ctx);
 lbm_status lbm_get_tuning(const lbm_ctx *ctx, int32_t lattice, int32_t *vec, int32_t *rows,
                           int32_t *warps, int32_t *stages);
 
+/* The form of the steps that take no sample, beside the shape of those that do:
+ * 0: the same shape; 1: the direct kernel in strips of 32 vec columns and `rows`
+ * rows, `warps` strips to a block, where vec need not divide nx and rows may
+ * be 1 to 4096 (D2Q7: even); 2: stretches of them as resident launches
+ * (lbm_set_persistent) of clusters of `vec` blocks, single ones as 0.  The tuner
+ * chooses among them; lbm_set_plain_form pins one for every launch group, for
+ * tests and measurements, after lbm_set_tuning has fixed the shape (which also
+ * returns to form 0), and refuses what a group cannot run.  lbm_get_plain_form
+ * reports lattice `lattice`'s (vec, rows and warps are 0 where they do not apply). */
+lbm_status lbm_set_plain_form(lbm_ctx *ctx, int32_t form, int32_t vec, int32_t rows, int32_t warps);
+lbm_status lbm_get_plain_form(const lbm_ctx *ctx, int32_t lattice, int32_t *form, int32_t *vec,
+                              int32_t *rows, int32_t *warps);
+
 /* CUDA-graph replay of lbm_step: 1 = capture each distinct step sequence once
  * and replay it (default), 0 = launch kernels directly. */
 lbm_status lbm_set_graphs(lbm_ctx *ctx, int32_t enabled);

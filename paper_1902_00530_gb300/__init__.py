@@ -221,6 +221,18 @@ class Simulation:
                                             ctypes.byref(s)))
         return v.value, r.value, w.value, s.value
 
+    def set_plain_form(self, form: int, vec: int = 0, rows: int = 0, warps: int = 0) -> None:
+        """Pin the form of steps that take no sample, after set_tuning(1, ...): 0 the
+        shape of sample steps, 1 a direct shape, 2 resident launches of clusters of vec blocks."""
+        self._check(self.lib.lbm_set_plain_form(self.ctx, form, vec, rows, warps))
+
+    def get_plain_form(self, lattice: int = 0) -> tuple:
+        """(form, vec, rows, warps) of the steps that take no sample."""
+        f, v, r, w = ctypes.c_int32(), ctypes.c_int32(), ctypes.c_int32(), ctypes.c_int32()
+        self._check(self.lib.lbm_get_plain_form(self.ctx, lattice, ctypes.byref(f), ctypes.byref(v), ctypes.byref(r),
+                                                ctypes.byref(w)))
+        return f.value, v.value, r.value, w.value
+
     def set_graphs(self, enabled: bool) -> None:
         self._check(self.lib.lbm_set_graphs(self.ctx, 1 if enabled else 0))
 

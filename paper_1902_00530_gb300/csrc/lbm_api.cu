@@ -882,7 +882,8 @@ void choose(GroupHost &g, const Choice &ch)
 }
 
 // The resident launch's plan for a group: the cluster size (blocks per
-// lattice) with the least estimated time per step, if any fits.  A step takes
+// lattice; `only` that one if it is not 0) with the least estimated time per
+// step, if any fits.  A step takes
 // a latency (barrier, one pass of dependent arithmetic) plus the sites an SM
 // has to update, in waves of the clusters that fit the GPU at once.  In SM
 // cycles, RES_STEP_CYCLES and RES_SITE_CYCLES stand for the latency of a step
@@ -891,7 +892,7 @@ void choose(GroupHost &g, const Choice &ch)
 // 180 x 60; only their order decides, waves first, then the cluster size).
 constexpr double RES_STEP_CYCLES = 1000.0, RES_SITE_CYCLES = 4.0;
 
-bool plan_resident(const lbm_ctx *c, GroupHost &g)
+bool plan_resident(const lbm_ctx *c, GroupHost &g, int only = 0)
 {
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return false;
@@ -901,7 +902,7 @@ bool plan_resident(const lbm_ctx *c, GroupHost &g)
     const int nl = (int)g.members.size();
     double best = 1e30;
     long long prev_sites = -1;
-    for (int C = 1; C <= 16; ++C) {
+    for (int C = only ? only : 1; C <= (only ? only : 16); ++C) {
         if (min_ny / C < resident_halo(g.model)) break;
         size_t smem = 0;
         long long sites = 0;
@@ -1796,6 +1797,54 @@ lbm_status lbm_get_tuning(const lbm_ctx *c, int32_t lattice, int32_t *vec, int32
     *rows = g.rows;
     *warps = g.warps;
     *stages = g.stages;
+    return LBM_OK;
+}
+
+lbm_status lbm_set_plain_form(lbm_ctx *c, int32_t form, int32_t vec, int32_t rows, int32_t warps)
+{
+    lbm_status st = require_ready(c, false);
+    if (st != LBM_OK) return st;
+    if (c->tune_mode != 1) return fail(c, LBM_ERR_INVALID_ARG, "fix the shape of sample steps first (lbm_set_tuning)");
+    if (form < 0 || form > 2) return fail(c, LBM_ERR_INVALID_ARG, "form must be 0, 1 or 2");
+    if (form == 1) {
+        if (rows < 1 || rows > 4096) return fail(c, LBM_ERR_INVALID_ARG, "rows must be in [1, 4096]");
+        if (warps < 1 || warps > 8) return fail(c, LBM_ERR_INVALID_ARG, "warps must be in [1, 8]");
+        for (auto &g : c->groups) {
+            if (!direct_ok(c, g))
+                return fail(c, LBM_ERR_INVALID_ARG, "direct kernel needs q ny pitch <= 2^32 elements");
+            if (g.q == 7 && rows % 2) return fail(c, LBM_ERR_INVALID_ARG, "D2Q7 strips need an even number of rows");
+            if (!allowed_vec(g.storage, vec))
+                return fail(c, LBM_ERR_INVALID_ARG, "vec not available for this storage");
+        }
+    }
+    if (form == 2) {
+        if (c->persist_mode != 2) return fail(c, LBM_ERR_INVALID_ARG, "the resident launch needs launch form mode 2");
+        if (vec < 1 || vec > 16) return fail(c, LBM_ERR_INVALID_ARG, "clusters have 1 to 16 blocks");
+        const std::vector<GroupHost> before = c->groups;
+        for (auto &g : c->groups)
+            if (!plan_resident(c, g, vec)) {
+                c->groups = before;
+                return fail(c, LBM_ERR_INVALID_ARG, "a cluster of this size does not hold every lattice");
+            }
+    }
+    for (auto &g : c->groups) {
+        g.plain = form == 1 ? Shape{vec, rows, warps, 0} : Shape{0, 0, 0, 0};
+        g.resident = form == 2;
+    }
+    drop_graphs(c);
+    return upload_descs(c);
+}
+
+lbm_status lbm_get_plain_form(const lbm_ctx *c, int32_t lattice, int32_t *form, int32_t *vec, int32_t *rows,
+                              int32_t *warps)
+{
+    if (!c || !form || !vec || !rows || !warps || lattice < 0 || lattice >= (int32_t)c->lats.size())
+        return LBM_ERR_INVALID_ARG;
+    const GroupHost &g = c->groups[c->lats[lattice].group];
+    *form = resident_ok(c, g) ? 2 : (g.plain.rows > 0 ? 1 : 0);
+    *vec = *form == 2 ? g.res_cluster : (*form == 1 ? g.plain.vec : 0);
+    *rows = *form == 1 ? g.plain.rows : 0;
+    *warps = *form == 1 ? g.plain.warps : 0;
     return LBM_OK;
 }
 
