@@ -206,7 +206,7 @@ __global__ void __maxnreg__(staged_max_regs<VEC>()) step_staged_kernel_q7(const 
     constexpr bool MIPS = (MODEL == MODEL_MIPS);
     const int q_first_row = MIPS ? y_begin - 1 : y_begin;
     const int nq = (y_end - y_begin) + (MIPS ? 2 : 0);
-    auto stage_ptr = [&](RingPos r) { return ring + (size_t)r.slot() * stage_elems; };
+    auto stage_ptr = [&](RingPos<VEC> r) { return ring + (size_t)r.slot() * stage_elems; };
     bool ok = true;
     auto fail = [&]() {
         ok = false;
@@ -223,7 +223,7 @@ __global__ void __maxnreg__(staged_max_regs<VEC>()) step_staged_kernel_q7(const 
 
     // Row q is consumed by this warp; warp 0 refills its buffer with row q + S
     // once every warp has (a single warp needs no barrier for that).
-    auto release = [&](RingPos r) {
+    auto release = [&](RingPos<VEC> r) {
         __syncwarp();
         if (blk.nact == 1) {  // a single warp: its own reads are all there is to wait for
             if (ok && issued < nq) issue(r.slot());
@@ -235,7 +235,7 @@ __global__ void __maxnreg__(staged_max_regs<VEC>()) step_staged_kernel_q7(const 
             else issue(r.slot());
         }
     };
-    auto wait_row = [&](RingPos r) {
+    auto wait_row = [&](RingPos<VEC> r) {
         if (ok && !stage_wait(&full[r.slot()], r.phase())) fail();
         return ok;
     };
@@ -246,7 +246,7 @@ __global__ void __maxnreg__(staged_max_regs<VEC>()) step_staged_kernel_q7(const 
 
     float rm[VEC + 2], rc[VEC + 2], rn[VEC + 2];
     int y_next = y_begin;  // row to update next, and its place in the ring
-    RingPos at{0};
+    RingPos<VEC> at{};
     if constexpr (MIPS) {
         if (wait_row(at)) {
             stage_density_window7<ST, VEC, 1>(stage_ptr(at), sg, b, sh, lane, rm);  // row y_begin-1: odd
@@ -262,7 +262,7 @@ __global__ void __maxnreg__(staged_max_regs<VEC>()) step_staged_kernel_q7(const 
     // one row of parity P; returns false if a wait gave up
     auto do_row = [&](auto parity, int y) -> bool {
         constexpr int P = decltype(parity)::value;
-        const RingPos cur = at;
+        const RingPos<VEC> cur = at;
         at = at.next(S);
         float f[7][VEC];
         if constexpr (CONV) {
@@ -341,7 +341,7 @@ __global__ void __maxnreg__(staged_max_regs<VEC>()) step_staged_kernel_q7(const 
     if (leader) {
         // the copies warp 0 issued must land before the block's shared memory is
         // released: wait for the rows it has not waited for itself (bounded)
-        RingPos r = MIPS ? at.next(S) : at;
+        RingPos<VEC> r = MIPS ? at.next(S) : at;
         for (int qq = (y_next - y_begin) + (MIPS ? 2 : 0); qq < issued; ++qq, r = r.next(S)) (void)stage_wait(&full[r.slot()], r.phase());
     }
     if (!ok) return;

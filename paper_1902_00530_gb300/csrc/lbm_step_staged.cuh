@@ -292,14 +292,27 @@ template <int VEC> constexpr int staged_max_regs()
 
 // A row's place in the ring: its buffer and the phase parity of the buffer's
 // barriers.  Both advance by counting: row q's are q mod S and (q / S) mod 2, but S is
-// not a constant, and a division is a chain of a dozen instructions.  One word, since
-// the kernels of 8-site vectors have no register to spare.
-struct RingPos {
+// not a constant, and a division is a chain of a dozen instructions (4096^2 MIPS FP32
+// 322 -> 314 instructions per site).  The kernels of 8-site vectors, which spill, hold both in
+// one word (4096^2 passive FP16, shape 8,32,4,4: 187 us per step in two, 171 in one); the
+// others do not need to and save the instructions that take it apart.
+template <bool ONE_WORD> struct RingPosForm {
+    int s;
+    uint32_t p;
+    __device__ __forceinline__ int slot() const { return s; }
+    __device__ __forceinline__ uint32_t phase() const { return p; }
+    __device__ __forceinline__ RingPosForm next(int S) const
+    {
+        return s + 1 == S ? RingPosForm{0, p ^ 1u} : RingPosForm{s + 1, p};
+    }
+};
+template <> struct RingPosForm<true> {
     int v;  // 2 slot + phase
     __device__ __forceinline__ int slot() const { return v >> 1; }
     __device__ __forceinline__ uint32_t phase() const { return (uint32_t)v & 1u; }
-    __device__ __forceinline__ RingPos next(int S) const { return RingPos{v + 2 < 2 * S ? v + 2 : (v & 1) ^ 1}; }
+    __device__ __forceinline__ RingPosForm next(int S) const { return RingPosForm{v + 2 < 2 * S ? v + 2 : (v & 1) ^ 1}; }
 };
+template <int VEC> using RingPos = RingPosForm<(VEC > 4)>;
 
 // The block's place in its lattice: strip row sy, first strip column sx0, and
 // the number of its warps whose strips lie inside the lattice (at least 1).
@@ -376,7 +389,7 @@ __global__ void __maxnreg__(staged_max_regs<VEC>()) step_staged_kernel(const Ste
     constexpr bool MIPS = (MODEL == MODEL_MIPS);
     const int q_first_row = MIPS ? y_begin - 1 : y_begin;
     const int nq = (y_end - y_begin) + (MIPS ? 2 : 0);
-    auto stage_ptr = [&](RingPos r) { return ring + (size_t)r.slot() * stage_elems; };
+    auto stage_ptr = [&](RingPos<VEC> r) { return ring + (size_t)r.slot() * stage_elems; };
     bool ok = true;
     auto fail = [&]() {
         ok = false;
@@ -394,7 +407,7 @@ __global__ void __maxnreg__(staged_max_regs<VEC>()) step_staged_kernel(const Ste
     // Row q is consumed: every lane of the warp has finished its reads, and the
     // warp tells warp 0, which refills the buffer with row q + S once all warps
     // have done so.
-    auto release = [&](RingPos r) {
+    auto release = [&](RingPos<VEC> r) {
         __syncwarp();
         if (blk.nact == 1) {  // a single warp: its own reads are all there is to wait for
             if (ok && issued < nq) issue(r.slot());
@@ -406,7 +419,7 @@ __global__ void __maxnreg__(staged_max_regs<VEC>()) step_staged_kernel(const Ste
             else issue(r.slot());
         }
     };
-    auto wait_row = [&](RingPos r) {
+    auto wait_row = [&](RingPos<VEC> r) {
         if (ok && !stage_wait(&full[r.slot()], r.phase())) fail();
         return ok;
     };
@@ -420,7 +433,7 @@ __global__ void __maxnreg__(staged_max_regs<VEC>()) step_staged_kernel(const Ste
     // released one row earlier.
     float rm[VEC + 2], rc[VEC + 2], rn[VEC + 2];
     int q = 0;            // row to update next, and its place in the ring
-    RingPos at{0};
+    RingPos<VEC> at{};
     if constexpr (MIPS) {
         if (wait_row(at)) {
             stage_density_window<ST, VEC>(stage_ptr(at), sg, b, sh, lane, rm);
@@ -435,7 +448,7 @@ __global__ void __maxnreg__(staged_max_regs<VEC>()) step_staged_kernel(const Ste
     }
 
     for (int y = y_begin; y < y_end && ok; ++y) {
-        const RingPos cur = at;
+        const RingPos<VEC> cur = at;
         at = at.next(S);
         float f[9][VEC];
         if constexpr (CONV) {
@@ -505,7 +518,7 @@ __global__ void __maxnreg__(staged_max_regs<VEC>()) step_staged_kernel(const Ste
         // every copy warp 0 issued must land before the block's shared memory
         // is released: wait for the rows it has not waited for itself (the
         // latest phase of each of their buffers; bounded)
-        RingPos r = MIPS ? at.next(S) : at;
+        RingPos<VEC> r = MIPS ? at.next(S) : at;
         for (int qq = q + (MIPS ? 1 : 0); qq < issued; ++qq, r = r.next(S)) (void)stage_wait(&full[r.slot()], r.phase());
     }
     if (!ok) return;
