@@ -691,14 +691,16 @@ __device__ __forceinline__ void observe_moments(const float rv[VEC], const float
             o.wide = true;
         }
     }
-    double row = pair_value(pair_warp_sum(rs));
+    rs = pair_warp_sum(rs);
     if (__any_sync(FULL, wide)) {
         double w = 0.0;
 #pragma unroll
         for (int j = 0; j < VEC; ++j) w += wide ? (double)rv[j] : 0.0;
-        row += warp_sum_f64(w);
+        w = warp_sum_f64(w);
+        if (lane == 0) *row_out = pair_value(rs) + w;
+    } else if (lane == 0) {  // FP64 in the one lane: in all it would be the row's longest latency
+        *row_out = pair_value(rs);
     }
-    if (lane == 0) *row_out = row;
 }
 
 // The same for a stored D2Q9 row.
@@ -723,24 +725,29 @@ __device__ __forceinline__ void observe_flush(double *colp, double *scal, int nx
                                               bool valid, const ObserveSums<VEC> &o, int lane)
 {
     Pair rho{0.f, 0.f};
-    double far = 0.0;  // what lies outside the pairs
 #pragma unroll
     for (int j = 0; j < VEC; ++j) pair_add(rho, o.col[j]);
+    double *const cols = colp + (size_t)sy * nx + x0;
+    const bool any_wide = __any_sync(FULL, o.wide);
+    double far = 0.0;  // what lies outside the pairs
+    if (any_wide) {
+#pragma unroll
+        for (int j = 0; j < VEC; ++j) far += o.wide ? cols[j] : 0.0;
+        far = warp_sum_f64(far);
+    }
     if (valid) {
-        double *const cols = colp + (size_t)sy * nx + x0;
 #pragma unroll
         for (int j = 0; j < VEC; ++j) {
-            const double w = o.wide ? cols[j] : 0.0;
-            far += w;
-            cols[j] = pair_value(o.col[j]) + w;
+            const double c = pair_value(o.col[j]);
+            if (o.wide) cols[j] += c;
+            else cols[j] = c;
         }
     }
     const Pair v[4] = {pair_warp_sum(rho), pair_warp_sum(o.jx), pair_warp_sum(o.jy), pair_warp_sum(o.aj)};
     const double r2 = warp_sum_f64((pair_value(o.r2) + (double)o.r2m) + o.r2d);
-    if (__any_sync(FULL, o.wide)) far = warp_sum_f64(far);
     if (lane == 0) {
         double *out = scal + (size_t)s * 5;
-        out[0] = pair_value(v[0]) + far;
+        out[0] = any_wide ? pair_value(v[0]) + far : pair_value(v[0]);
         out[1] = pair_value(v[1]);
         out[2] = pair_value(v[2]);
         out[3] = r2;
