@@ -609,8 +609,8 @@ __device__ __forceinline__ Pair pair_warp_sum(Pair a)
 }
 
 // The pairs hold FP32's range, and a strip's sum has up to 2^20 terms (4096 rows
-// of 8 sites in 32 lanes): densities from PAIR_MAX on are summed in FP64, in the strip's
-// own column partials, which only its lane writes.  (Sums of j need no such
+// of 8 sites in 32 lanes): a strip with a density from PAIR_MAX on is summed again,
+// in FP64, from its stored populations (observe_wide).  (Sums of j need no such
 // form: from |j| = 2^64 on |j|^2 is infinite, which the finaliser reports.)
 // rho^2 = p + fma(r, r, -p) has 48 bits itself, and the variance is the small
 // difference of two such sums, so its sum is three words (h + l + m).  That holds
@@ -624,7 +624,7 @@ template <int VEC> struct ObserveSums {
     Pair col[VEC], jx, jy, r2, aj;
     float r2m;
     double r2d;
-    bool wide;  // the lane has column sums in FP64 too
+    bool wide;  // a density beyond the pairs: the sums of rho are void
     __device__ __forceinline__ void clear()
     {
 #pragma unroll
@@ -643,28 +643,29 @@ __device__ __forceinline__ double warp_sum_f64(double v)
 }
 
 // Add one stored row (sites x0..x0+VEC-1) from its moments rho and j = rho u,
-// and write the row's density total over the warp.  cols: the lane's column partials
-// (see PAIR_MAX).  |j|, a sum of magnitudes, is summed in FP32 over the lane's sites
-// of the row.  Lattice-independent.
+// and write the row's density total over the warp.  |j|, a sum of magnitudes,
+// is summed in FP32 over the lane's sites of the row.  Lattice-independent.
 template <int VEC>
 __device__ __forceinline__ void observe_moments(const float rv[VEC], const float jxv[VEC], const float jyv[VEC],
-                                                bool valid, ObserveSums<VEC> &o, double *cols, double *row_out, int lane)
+                                                bool valid, ObserveSums<VEC> &o, double *row_out, int lane)
 {
     Pair rs{0.f, 0.f};
-    bool wide = false;
     if (valid) {
         float js = 0.f;
-        bool squares = true;
+        bool in_range = true;
 #pragma unroll
         for (int j = 0; j < VEC; ++j) {
             const float r = rv[j], jx = jxv[j], jy = jyv[j];
+            pair_add(o.col[j], r);
             pair_add(o.jx, jx);
             pair_add(o.jy, jy);
-            squares = squares && r > SQUARE_MIN && r < SQUARE_MAX;
+            in_range = in_range && r > SQUARE_MIN && r < SQUARE_MAX;
             js += sqrtf(jx * jx + jy * jy);
+            if (j == 0) rs.h = r;
+            else pair_add(rs, r);
         }
         pair_add(o.aj, js);
-        if (squares) {
+        if (in_range) {
 #pragma unroll
             for (int j = 0; j < VEC; ++j) {
                 const float p = __fmul_rn(rv[j], rv[j]);
@@ -675,38 +676,18 @@ __device__ __forceinline__ void observe_moments(const float rv[VEC], const float
 #pragma unroll
             for (int j = 0; j < VEC; ++j) {
                 o.r2d = __fma_rn((double)rv[j], (double)rv[j], o.r2d);
-                wide = wide || !(fabsf(rv[j]) < PAIR_MAX);
+                o.wide = o.wide || !(fabsf(rv[j]) < PAIR_MAX);
             }
-        }
-        if (!wide) {
-#pragma unroll
-            for (int j = 0; j < VEC; ++j) {
-                pair_add(o.col[j], rv[j]);
-                if (j == 0) rs.h = rv[j];
-                else pair_add(rs, rv[j]);
-            }
-        } else {
-#pragma unroll
-            for (int j = 0; j < VEC; ++j) cols[j] = (o.wide ? cols[j] : 0.0) + (double)rv[j];
-            o.wide = true;
         }
     }
     rs = pair_warp_sum(rs);
-    if (__any_sync(FULL, wide)) {
-        double w = 0.0;
-#pragma unroll
-        for (int j = 0; j < VEC; ++j) w += wide ? (double)rv[j] : 0.0;
-        w = warp_sum_f64(w);
-        if (lane == 0) *row_out = pair_value(rs) + w;
-    } else if (lane == 0) {  // FP64 in the one lane: in all it would be the row's longest latency
-        *row_out = pair_value(rs);
-    }
+    if (lane == 0) *row_out = pair_value(rs);
 }
 
 // The same for a stored D2Q9 row.
 template <int VEC>
-__device__ __forceinline__ void observe_row(const float g[9][VEC], bool valid, ObserveSums<VEC> &o, double *cols,
-                                            double *row_out, int lane)
+__device__ __forceinline__ void observe_row(const float g[9][VEC], bool valid, ObserveSums<VEC> &o, double *row_out,
+                                            int lane)
 {
     float rv[VEC], jxv[VEC], jyv[VEC];
 #pragma unroll
@@ -715,43 +696,73 @@ __device__ __forceinline__ void observe_row(const float g[9][VEC], bool valid, O
         jxv[j] = (g[1][j] + g[5][j] + g[8][j]) - (g[3][j] + g[6][j] + g[7][j]);
         jyv[j] = (g[2][j] + g[5][j] + g[6][j]) - (g[4][j] + g[7][j] + g[8][j]);
     }
-    observe_moments<VEC>(rv, jxv, jyv, valid, o, cols, row_out, lane);
+    observe_moments<VEC>(rv, jxv, jyv, valid, o, row_out, lane);
+}
+
+// The sums of rho of a strip (rows y_begin .. y_end-1) of stored populations in FP64: its
+// column and row partials, and its total in every lane.
+template <int Q, int ST, int VEC>
+__device__ __noinline__ double observe_wide(const typename Store<ST>::T *base, size_t plane, int pitch, int y_begin,
+                                            int y_end, int x0, bool valid, const Shift3 &sh, double *cols, double *rows,
+                                            int lane)
+{
+    double col[VEC], total = 0.0;
+#pragma unroll
+    for (int j = 0; j < VEC; ++j) col[j] = 0.0;
+    for (int y = y_begin; y < y_end; ++y) {
+        double row = 0.0;
+        if (valid) {
+#pragma unroll
+            for (int j = 0; j < VEC; ++j) {
+                const typename Store<ST>::T *p = base + (size_t)y * pitch + x0 + j;
+                float f[9];
+#pragma unroll
+                for (int i = 0; i < Q; ++i) f[i] = load_one<ST>(p + i * plane, sh.of(Q, i));
+                float r = __fadd_rn(__fadd_rn(f[0], f[1]), __fadd_rn(f[2], f[3]));
+                if constexpr (Q == 7) r = __fadd_rn(r, __fadd_rn(__fadd_rn(f[4], f[5]), f[6]));
+                else r = __fadd_rn(__fadd_rn(r, __fadd_rn(__fadd_rn(f[4], f[5]), __fadd_rn(f[6], f[7]))), f[8]);
+                col[j] += (double)r;
+                row += (double)r;
+            }
+        }
+        row = warp_sum_f64(row);
+        if (lane == 0) rows[y] = row;
+        total += row;
+    }
+    if (valid) {
+#pragma unroll
+        for (int j = 0; j < VEC; ++j) cols[j] = col[j];
+    }
+    return total;
 }
 
 // Write the strip's column sums and its five scalar sums (rho, j_x, j_y, rho^2,
-// |j|).
-template <int VEC>
+// |j|).  wide(cols) is observe_wide of the strip.
+template <int VEC, typename Wide>
 __device__ __forceinline__ void observe_flush(double *colp, double *scal, int nx, int s, int sy, int x0,
-                                              bool valid, const ObserveSums<VEC> &o, int lane)
+                                              bool valid, const ObserveSums<VEC> &o, int lane, Wide wide)
 {
     Pair rho{0.f, 0.f};
 #pragma unroll
     for (int j = 0; j < VEC; ++j) pair_add(rho, o.col[j]);
     double *const cols = colp + (size_t)sy * nx + x0;
-    const bool any_wide = __any_sync(FULL, o.wide);
-    double far = 0.0;  // what lies outside the pairs
-    if (any_wide) {
-#pragma unroll
-        for (int j = 0; j < VEC; ++j) far += o.wide ? cols[j] : 0.0;
-        far = warp_sum_f64(far);
-    }
     if (valid) {
 #pragma unroll
-        for (int j = 0; j < VEC; ++j) {
-            const double c = pair_value(o.col[j]);
-            if (o.wide) cols[j] += c;
-            else cols[j] = c;
-        }
+        for (int j = 0; j < VEC; ++j) cols[j] = pair_value(o.col[j]);
     }
     const Pair v[4] = {pair_warp_sum(rho), pair_warp_sum(o.jx), pair_warp_sum(o.jy), pair_warp_sum(o.aj)};
     const double r2 = warp_sum_f64((pair_value(o.r2) + (double)o.r2m) + o.r2d);
+    double *const out = scal + (size_t)s * 5;
     if (lane == 0) {
-        double *out = scal + (size_t)s * 5;
-        out[0] = any_wide ? pair_value(v[0]) + far : pair_value(v[0]);
+        out[0] = pair_value(v[0]);
         out[1] = pair_value(v[1]);
         out[2] = pair_value(v[2]);
         out[3] = r2;
         out[4] = pair_value(v[3]);
+    }
+    if (__any_sync(FULL, o.wide)) {
+        const double total = wide(cols);
+        if (lane == 0) out[0] = total;
     }
 }
 
@@ -891,7 +902,7 @@ __device__ __forceinline__ void direct_strip(const StepArgs &a, const LatDesc *d
 #pragma unroll
                 for (int j = 0; j < VEC; ++j)
                     g[i][j] = Store<ST>::get(Store<ST>::put(out[i][j], sh.q9(i)), sh.q9(i));
-            observe_row<VEC>(g, valid, obs, dp->colp + (size_t)sy * nx + x0, dp->rowp + (size_t)sx * ny + y, lane);
+            observe_row<VEC>(g, valid, obs, dp->rowp + (size_t)sx * ny + y, lane);
         }
         if constexpr (MODEL == MODEL_MIPS) {
 #pragma unroll
@@ -902,7 +913,10 @@ __device__ __forceinline__ void direct_strip(const StepArgs &a, const LatDesc *d
         }
         if (!SAMPLE && RO && y + 1 == y_end) allow_dependents();
     }
-    if constexpr (SAMPLE) observe_flush<VEC>(dp->colp, dp->scal, nx, s, sy, x0, valid, obs, lane);
+    if constexpr (SAMPLE) observe_flush<VEC>(dp->colp, dp->scal, nx, s, sy, x0, valid, obs, lane, [&](double *cols) {
+            return observe_wide<9, ST, VEC>(dst, plane, pitch, y_begin, y_end, x0, valid, sh, cols,
+                                           dp->rowp + (size_t)sx * ny, lane);
+        });
 }
 
 template <int MODEL, int ST, int VEC, bool SAMPLE, int NOISE, bool RAGGED>
@@ -970,9 +984,12 @@ __global__ void __launch_bounds__(256) observe_kernel(const StepArgs a)
             }
         }
         fetch(min(y + 1, y_end - 1));  // in flight during this row's sums and shuffles
-        observe_row<VEC>(g, valid, obs, dp->colp + (size_t)sy * nx + x0, dp->rowp + (size_t)sx * ny + y, lane);
+        observe_row<VEC>(g, valid, obs, dp->rowp + (size_t)sx * ny + y, lane);
     }
-    observe_flush<VEC>(dp->colp, dp->scal, nx, s, sy, x0, valid, obs, lane);
+    observe_flush<VEC>(dp->colp, dp->scal, nx, s, sy, x0, valid, obs, lane, [&](double *cols) {
+            return observe_wide<9, ST, VEC>(src, plane, pitch, y_begin, y_end, x0, valid, sh, cols,
+                                           dp->rowp + (size_t)sx * ny, lane);
+        });
 }
 
 }  // namespace lbm

@@ -247,7 +247,7 @@ __device__ __forceinline__ void noise_u7(uint32_t x, uint32_t y, uint32_t t, uin
 
 template <int VEC>
 __device__ __forceinline__ void observe_row7(const float g[7][VEC], bool valid, ObserveSums<VEC> &o,
-                                             double *cols, double *row_out, int lane)
+                                             double *row_out, int lane)
 {
     float rv[VEC], jxv[VEC], jyv[VEC];
 #pragma unroll
@@ -256,7 +256,7 @@ __device__ __forceinline__ void observe_row7(const float g[7][VEC], bool valid, 
         jxv[j] = (g[1][j] - g[4][j]) + 0.5f * ((g[2][j] + g[6][j]) - (g[3][j] + g[5][j]));
         jyv[j] = Q7_HALF_SQRT3 * ((g[2][j] + g[3][j]) - (g[5][j] + g[6][j]));
     }
-    observe_moments<VEC>(rv, jxv, jyv, valid, o, cols, row_out, lane);
+    observe_moments<VEC>(rv, jxv, jyv, valid, o, row_out, lane);
 }
 
 // Per-warp state of the row walk.
@@ -271,7 +271,7 @@ template <int MODEL, int ST, int VEC, bool SAMPLE, int P, bool RAGGED, bool RO>
 __device__ __forceinline__ void q7_row(Q7Walk<VEC> &w, int y, const typename Store<ST>::T *src,
                                        typename Store<ST>::T *dst, size_t plane, int nx, int ny, int pitch, int x0,
                                        bool valid, bool last, int lane, const Shift3 &sh, const SiteParams &d, bool noise,
-                                       uint32_t t, uint32_t id, const uint32_t *rk, double *colp, double *rowp)
+                                       uint32_t t, uint32_t id, const uint32_t *rk, double *rowp)
 {
     float fn[7][VEC];
     const bool partial = RAGGED && valid && x0 + VEC > nx;
@@ -314,7 +314,7 @@ __device__ __forceinline__ void q7_row(Q7Walk<VEC> &w, int y, const typename Sto
 #pragma unroll
             for (int j = 0; j < VEC; ++j)
                 g[i][j] = Store<ST>::get(Store<ST>::put(out[i][j], sh.q7(i)), sh.q7(i));
-        observe_row7<VEC>(g, valid, w.obs, colp, rowp + y, lane);
+        observe_row7<VEC>(g, valid, w.obs, rowp + y, lane);
     }
     if constexpr (MODEL == MODEL_MIPS) {
 #pragma unroll
@@ -354,7 +354,7 @@ __device__ __forceinline__ void direct_strip_q7(const StepArgs &a, const LatDesc
     const T *src = reinterpret_cast<const T *>(dp->f[src_buf]);
     T *dst = reinterpret_cast<T *>(dp->f[src_buf ^ 1]);
     const bool noise = NOISE == 2 ? d.sigma_q > 0.f : NOISE == 1;  // as in step_kernel
-    double *colp = dp->colp + (size_t)sy * nx + x0, *rowp = dp->rowp + (size_t)sx * ny;
+    double *rowp = dp->rowp + (size_t)sx * ny;
 
     Q7Walk<VEC> w;
     if constexpr (SAMPLE) w.obs.clear();
@@ -371,12 +371,15 @@ __device__ __forceinline__ void direct_strip_q7(const StepArgs &a, const LatDesc
     }
     for (int y = y_begin; y < y_end; y += 2) {
         q7_row<MODEL, ST, VEC, SAMPLE, 0, RAGGED, RO>(w, y, src, dst, plane, nx, ny, pitch, x0, valid, last, lane, sh, d, noise,
-                                          t, id, a.rk, colp, rowp);
+                                          t, id, a.rk, rowp);
         q7_row<MODEL, ST, VEC, SAMPLE, 1, RAGGED, RO>(w, y + 1, src, dst, plane, nx, ny, pitch, x0, valid, last, lane, sh, d,
-                                          noise, t, id, a.rk, colp, rowp);
+                                          noise, t, id, a.rk, rowp);
         if (!SAMPLE && RO && y + 2 >= y_end) allow_dependents();
     }
-    if constexpr (SAMPLE) observe_flush<VEC>(dp->colp, dp->scal, nx, s, sy, x0, valid, w.obs, lane);
+    if constexpr (SAMPLE) observe_flush<VEC>(dp->colp, dp->scal, nx, s, sy, x0, valid, w.obs, lane, [&](double *cols) {
+            return observe_wide<7, ST, VEC>(dst, plane, pitch, y_begin, y_end, x0, valid, sh, cols,
+                                           dp->rowp + (size_t)sx * ny, lane);
+        });
 }
 
 template <int MODEL, int ST, int VEC, bool SAMPLE, int NOISE, bool RAGGED>
@@ -452,9 +455,12 @@ __global__ void __launch_bounds__(256) observe_kernel_q7(const StepArgs a)
             }
         }
         fetch(min(y + 1, y_end - 1));  // in flight during this row's sums and shuffles
-        observe_row7<VEC>(g, valid, obs, dp->colp + (size_t)sy * nx + x0, dp->rowp + (size_t)sx * ny + y, lane);
+        observe_row7<VEC>(g, valid, obs, dp->rowp + (size_t)sx * ny + y, lane);
     }
-    observe_flush<VEC>(dp->colp, dp->scal, nx, s, sy, x0, valid, obs, lane);
+    observe_flush<VEC>(dp->colp, dp->scal, nx, s, sy, x0, valid, obs, lane, [&](double *cols) {
+            return observe_wide<7, ST, VEC>(src, plane, pitch, y_begin, y_end, x0, valid, sh, cols,
+                                           dp->rowp + (size_t)sx * ny, lane);
+        });
 }
 
 }  // namespace lbm

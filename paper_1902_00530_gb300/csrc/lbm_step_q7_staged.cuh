@@ -322,7 +322,7 @@ __global__ void __maxnreg__(staged_max_regs<VEC>()) step_staged_kernel_q7(const 
 #pragma unroll
                 for (int j = 0; j < VEC; ++j)
                     g[i][j] = Store<ST>::get(Store<ST>::put(out[i][j], sh.q7(i)), sh.q7(i));
-            observe_row7<VEC>(g, valid, obs, dp->colp + (size_t)sy * nx + x0, rowp + y, lane);
+            observe_row7<VEC>(g, valid, obs, rowp + y, lane);
         }
         if constexpr (MIPS) {
 #pragma unroll
@@ -345,7 +345,10 @@ __global__ void __maxnreg__(staged_max_regs<VEC>()) step_staged_kernel_q7(const 
         for (int qq = (y_next - y_begin) + (MIPS ? 2 : 0); qq < issued; ++qq, r = r.next(S)) (void)stage_wait(&full[r.slot()], r.phase());
     }
     if (!ok) return;
-    if constexpr (SAMPLE) observe_flush<VEC>(dp->colp, dp->scal, nx, s, sy, x0, valid, obs, lane);
+    if constexpr (SAMPLE) observe_flush<VEC>(dp->colp, dp->scal, nx, s, sy, x0, valid, obs, lane, [&](double *cols) {
+            return observe_wide<7, ST, VEC>(dst, plane, pitch, y_begin, y_end, x0, valid, sh, cols,
+                                           dp->rowp + (size_t)sx * ny, lane);
+        });
 }
 
 template <int MODEL, int ST, int VEC, bool SAMPLE, int NOISE>

@@ -504,7 +504,7 @@ __global__ void __maxnreg__(staged_max_regs<VEC>()) step_staged_kernel(const Ste
 #pragma unroll
                 for (int j = 0; j < VEC; ++j)
                     g[i][j] = Store<ST>::get(Store<ST>::put(out[i][j], sh.q9(i)), sh.q9(i));
-            observe_row<VEC>(g, valid, obs, dp->colp + (size_t)sy * nx + x0, dp->rowp + (size_t)sx * ny + y, lane);
+            observe_row<VEC>(g, valid, obs, dp->rowp + (size_t)sx * ny + y, lane);
         }
         if constexpr (MIPS) {
 #pragma unroll
@@ -522,7 +522,10 @@ __global__ void __maxnreg__(staged_max_regs<VEC>()) step_staged_kernel(const Ste
         for (int qq = q + (MIPS ? 1 : 0); qq < issued; ++qq, r = r.next(S)) (void)stage_wait(&full[r.slot()], r.phase());
     }
     if (!ok) return;
-    if constexpr (SAMPLE) observe_flush<VEC>(dp->colp, dp->scal, nx, s, sy, x0, valid, obs, lane);
+    if constexpr (SAMPLE) observe_flush<VEC>(dp->colp, dp->scal, nx, s, sy, x0, valid, obs, lane, [&](double *cols) {
+            return observe_wide<9, ST, VEC>(dst, plane, pitch, y_begin, y_end, x0, valid, sh, cols,
+                                           dp->rowp + (size_t)sx * ny, lane);
+        });
 }
 
 
